@@ -33,17 +33,17 @@ def listed():
     return [
         # One image asked about on its own: visual tokens and prompt in, kept indices out, through the
         # encoder.  The smallest call: launches and the rounds' latency count.
-        _select("one image, encoded", "small", images=1, n_vis=576, n_txt=32, k_max=64, encode=True),
+        _select("one image encoded", "small", images=1, n_vis=576, n_txt=32, k_max=64, encode=True),
         # The batch of the headline workload, from a memory that an encoder of the user's own made, with
         # a STOP that ends some of the images early.
-        _select("batch, one token a round", "llava", images=16, n_vis=576, k_max=192, stop=True),
+        _select("batch of images", "llava", images=16, n_vis=576, k_max=192, stop=True),
         # Multi-tile images of 3,328 tokens, one episode each, five tokens a round: the keys of an
         # episode are larger than the shared memory of its cluster.
         _select("tiled images", "qwen", images=4, n_vis=3328, g=5, k_max=160),
         # A pointer decoder of two layers, images of uneven sizes.
         _select("two-layer pointer decoder", "llava", images=4, n_vis=576, k_max=64, dec_layers=2, ragged=True),
         # High-resolution images in groups of 576 candidates, encoded: the largest encoder call.
-        _select("any-resolution, encoded", "llava", images=8, n_vis=2880, n_txt=64, group=576, g=5, k_max=32,
+        _select("any-resolution encoded", "llava", images=8, n_vis=2880, n_txt=64, group=576, g=5, k_max=32,
                 encode=True),
         # The training-time forward: rollout with aggregates, soft top-k, noise gate.
         {"name": "training forward", "kind": "train", "dims": "llava", "images": 8, "n_vis": 576, "k_max": 96,
@@ -52,16 +52,16 @@ def listed():
         {"name": "gather and project", "kind": "project", "dims": "llava", "images": 16, "n_vis": 576, "n_txt": 48,
          "kept": 64},
         # The prefill of a pruned batch (about 1,800 packed tokens), writing the cache generation reads.
-        {"name": "prefill, pruned batch", "kind": "prefill", "dims": "llava", "seqs": 16, "tokens": 160,
+        {"name": "prefill pruned batch", "kind": "prefill", "dims": "llava", "seqs": 16, "tokens": 160,
          "ragged": True, "layers": 2, "kv": True},
         # Unpruned multi-tile prefixes with grouped-query heads and 3-D rotary positions.
-        {"name": "prefill, long", "kind": "prefill", "dims": "qwen", "seqs": 4, "tokens": 3424, "ragged": False,
+        {"name": "prefill long", "kind": "prefill", "dims": "qwen", "seqs": 4, "tokens": 3424, "ragged": False,
          "layers": 1, "kv": False},
         # One pruned image and its prompt: fewer rows than a tile, bound by the weights.
-        {"name": "prefill, one short", "kind": "prefill", "dims": "llava", "seqs": 1, "tokens": 97, "ragged": False,
+        {"name": "prefill one short", "kind": "prefill", "dims": "llava", "seqs": 1, "tokens": 97, "ragged": False,
          "layers": 2, "kv": True},
         # Generation after that batch's prefill: steps chained on the device.
-        {"name": "decode, batch", "kind": "decode", "dims": "llava", "seqs": 16, "context": 160, "ragged": True,
+        {"name": "decode batch", "kind": "decode", "dims": "llava", "seqs": 16, "context": 160, "ragged": True,
          "layers": 4, "steps": 4},
         # Visual tokens in, hidden states out: encoder, selection, gather, projector, prefill.
         {"name": "pipeline", "kind": "pipeline", "dims": "llava", "images": 4, "n_vis": 576, "n_txt": 48, "g": 1,
