@@ -463,7 +463,7 @@ sp_status plan_select(const sp_selector* s, const sp_select_in* in, SelPlan* p) 
 size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* out, Carve& cv,
                  void** parts) {
   const int D = s->cfg.D, h = s->cfg.h, F = s->cfg.enc_ffn;
-  float *P = nullptr, *R = nullptr, *Mall, *ZK, *XL, *QKVs;
+  float *P = nullptr, *R = nullptr, *ZK, *QKVs;
   void *Abf = nullptr, *QKV = nullptr, *O = nullptr, *F1 = nullptr;
   int* enc_cu = nullptr;
   void* gsk = nullptr;  // stream-K scratch of the encoder GEMMs (the precompute GEMMs run whole tiles)
@@ -479,9 +479,11 @@ size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* ou
   } else if (p.encoder) {
     R = cv.take<float>((size_t)p.T_enc * D);
   }
-  Mall = cv.take<float>((size_t)p.rows * D);
+  // (unused: the size that callers' workspaces and the allocation-free entry point's limit are checked
+  // against stays what it was when the memory and its LN1 were stored in fp32)
+  cv.take<float>((size_t)p.rows * D);
   ZK = cv.take<float>((size_t)p.rows * 2 * s->n_dec * h);
-  XL = cv.take<float>((size_t)p.rows * h);
+  cv.take<float>((size_t)p.rows * h);  // (unused, as above)
   QKVs = cv.take<float>((size_t)p.rows * 3 * h);
   void* Asp = cv.take<uint16_t>((size_t)p.rows * 3 * std::max(D, h));  // split operand of the precompute GEMMs
   int* order = (out && out->order) ? nullptr : cv.take<int>((size_t)p.E * SP_MAX_KMAX);
@@ -490,7 +492,7 @@ size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* ou
   float* dcache = s->n_dec > 1 ? cv.take<float>((size_t)p.E * (s->n_dec - 1) * (p.k_max + 1) * 2 * h) : nullptr;
   if (parts) {
     parts[0] = P; parts[1] = R; parts[2] = Abf; parts[3] = QKV; parts[4] = O; parts[5] = F1;
-    parts[6] = enc_cu; parts[7] = Mall; parts[8] = ZK; parts[9] = XL; parts[10] = QKVs;
+    parts[6] = enc_cu; parts[7] = nullptr; parts[8] = ZK; parts[9] = nullptr; parts[10] = QKVs;
     parts[11] = order; parts[12] = epc; parts[13] = gsk; parts[14] = Asp; parts[15] = dcache;
   }
   return cv.off;
@@ -519,16 +521,17 @@ sp_status run_encoder(const sp_selector* s, const sp_select_in* in, const SelPla
     ep.ldo = D;
     SP_CUDA(gemm_bf16(tE, p.ntxt, nullptr, s->Wp, D, ep, err, st, &gs), "text projection");
   }
-  SP_CUDA(assemble_encoder_input(p.bd, in->X, P, D, s->w.ln_text_g, s->w.ln_text_b, c.ln_eps, c.g_text, R,
-                                 p.T_enc, st), "encoder input");
-  SP_CUDA(write_enc_cu(p.bd, enc_cu, st), "encoder offsets");
+  SP_CUDA(assemble_encoder_input(p.bd, in->X, P, D, s->w.ln_text_g, s->w.ln_text_b, s->w.enc_ln1_g[0],
+                                 s->w.enc_ln1_b[0], c.ln_eps, c.g_text, R, Abf, p.T_enc, enc_cu, st),
+          "encoder input");
   CUtensorMap tA, tO, tF;
   if (!encode_tmap_bf16(&tA, Abf, p.T_enc, D, 128, &msg) || !encode_tmap_bf16(&tO, O, p.T_enc, D, 128, &msg) ||
       !encode_tmap_bf16(&tF, F1, p.T_enc, c.enc_ffn, 128, &msg))
     return fail(SP_ERR_CUDA, "%s", msg.c_str());
   const int nh = D / c.enc_head_dim;
   for (int l = 0; l < c.n_enc_layers; ++l) {
-    SP_CUDA(layernorm_f32(R, D, s->w.enc_ln1_g[l], s->w.enc_ln1_b[l], nullptr, Abf, D, p.T_enc, D, c.ln_eps, 1.f, st), "enc ln1");
+    if (l > 0)  // (the first block's LN1 was applied when its input was assembled)
+      SP_CUDA(layernorm_bf16(R, s->w.enc_ln1_g[l], s->w.enc_ln1_b[l], Abf, p.T_enc, D, c.ln_eps, st), "enc ln1");
     GemmEpi e1;
     e1.kind = EPI_BF16;
     e1.out = QKV;
@@ -542,7 +545,7 @@ sp_status run_encoder(const sp_selector* s, const sp_select_in* in, const SelPla
     e2.out = R;
     e2.ldo = D;
     SP_CUDA(gemm_bf16(tO, p.T_enc, nullptr, s->enc_o[l], D, e2, err, st, &gs), "enc o");
-    SP_CUDA(layernorm_f32(R, D, s->w.enc_ln2_g[l], s->w.enc_ln2_b[l], nullptr, Abf, D, p.T_enc, D, c.ln_eps, 1.f, st), "enc ln2");
+    SP_CUDA(layernorm_bf16(R, s->w.enc_ln2_g[l], s->w.enc_ln2_b[l], Abf, p.T_enc, D, c.ln_eps, st), "enc ln2");
     GemmEpi e3;
     e3.kind = EPI_GELU_BF16;
     e3.out = F1;
@@ -606,31 +609,23 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
   const GemmScratch gs = gemm_scratch_at(parts[13]);
   SP_CUDA(gemm_scratch_clear(gs, st), "GEMM scratch");
 
-  if (p.encoder && s->cfg.n_enc_layers > 0) {
+  // the candidate memory's rows go straight into the precompute's split operand:
+  // from the encoder, from X (no encoder blocks: H = X), or from the given H
+  const bool blocks = p.encoder && s->cfg.n_enc_layers > 0;
+  if (blocks) {
     rs = run_encoder(s, in, p, parts, err, st);
     if (rs != SP_OK) return rs;
-    SP_CUDA(gather_memory(p.bd, (float*)parts[1], nullptr, s->w.s_stop, s->w.s_start, (float*)parts[7], D, st), "memory");
-  } else if (p.encoder) {
-    // no encoder blocks: H = X (converted to fp32)
-    SP_CUDA(bf16_to_f32(in->X, (float*)parts[1], p.nvis, nullptr, D, st), "X to fp32");
-    BatchDesc flat = p.bd;
-    for (int b = 0; b <= in->B; ++b) flat.txt_off[b] = 0;
-    SP_CUDA(gather_memory(flat, (float*)parts[1], nullptr, s->w.s_stop, s->w.s_start, (float*)parts[7], D, st), "memory");
-  } else {
-    SP_CUDA(gather_memory(p.bd, nullptr, in->H, s->w.s_stop, s->w.s_start, (float*)parts[7], D, st), "memory");
   }
-  float* Mall = (float*)parts[7];
-  if (out->memory)
-    SP_CUDA(cudaMemcpyAsync(out->memory, Mall, (size_t)p.nvis * D * sizeof(float), cudaMemcpyDeviceToDevice, st),
-            "memory copy");
+  void* Asp = parts[14];
+  SP_CUDA(memory_split(p.bd, blocks ? (float*)parts[1] : nullptr, in->H, blocks ? nullptr : in->X, s->w.s_stop,
+                       s->w.s_start, Asp, out->memory, D, st),
+          "memory");
   float* ZK = (float*)parts[8];
-  float* XL = (float*)parts[9];
   float* QKVs = (float*)parts[10];
   // candidate precompute (fp32): [z | KT] = M [W_in; Wq_p^T Wk_p / sqrt h]^T, x = LN1(z),
   // [QS | KS | VT] = x [Wq_s / sqrt h; Wk_s; Wo_s Wv_s]^T
   // (fp32-accurate products on the bf16 tensor cores: three-way operand split)
   {
-    void* Asp = parts[14];
     std::string msg;
     CUtensorMap t1, t2;
     if (!encode_tmap_bf16(&t1, Asp, p.rows, 3 * D, 128, &msg) || !encode_tmap_bf16(&t2, Asp, p.rows, 3 * h, 128, &msg))
@@ -640,15 +635,13 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
     e1.out = ZK;
     e1.ldo = 2 * s->n_dec * h;
     const GemmASplit a1 = split3_a_map(D), a2 = split3_a_map(h);
-    SP_CUDA(split3_bf16(Mall, D, p.rows, D, Asp, st), "precompute split 1");
     SP_CUDA(gemm_bf16(t1, p.rows, nullptr, s->P1, 2 * s->n_dec * h, e1, err, st, nullptr, &a1), "precompute 1");
-    SP_CUDA(layernorm_f32(ZK, 2 * s->n_dec * h, s->pre_ln1_g, s->pre_ln1_b, XL, nullptr, h, p.rows, h, s->cfg.ln_eps,
-                          1.f, st), "ln1");
+    SP_CUDA(layernorm_split(ZK, 2 * s->n_dec * h, s->pre_ln1_g, s->pre_ln1_b, Asp, p.rows, h, s->cfg.ln_eps, st),
+            "ln1");
     GemmEpi e2;
     e2.kind = EPI_F32;
     e2.out = QKVs;
     e2.ldo = 3 * h;
-    SP_CUDA(split3_bf16(XL, h, p.rows, h, Asp, st), "precompute split 2");
     SP_CUDA(gemm_bf16(t2, p.rows, nullptr, s->P2, 3 * h, e2, err, st, nullptr, &a2), "precompute 2");
   }
 

@@ -151,8 +151,13 @@ cudaError_t gemm_bf16(const CUtensorMap& A, int M_cap, const int* M_dev, const G
                       const CUtensorMap* A16 = nullptr, const int* a_rows = nullptr);
 
 // ------------------------------------------------------------- candidate precompute
-// out [rows, 3K] bf16 = the three bf16 parts of x [rows, K] (fp32, row stride ldx).
-cudaError_t split3_bf16(const float* x, int ldx, int rows, int K, void* out, cudaStream_t st);
+// The candidate memory [visual rows of H, of X (bf16) or of the encoder's R; s_stop; s_start] as its three bf16
+// parts, out [rows, 3D]; memory (may be NULL) receives the visual rows in fp32.
+cudaError_t memory_split(const BatchDesc& bd, const float* R, const float* H, const void* X, const float* s_stop,
+                         const float* s_start, void* out, float* memory, int D, cudaStream_t st);
+// LN of fp32 rows (d <= 1,024, ldx apart) as their three bf16 parts, out [rows, 3d].
+cudaError_t layernorm_split(const float* x, int ldx, const float* gain, const float* bias, void* out, int rows, int d,
+                            float eps, cudaStream_t st);
 // out [N, 6K] bf16 = the weight segments b0 b1 b0 b2 b1 b0 of w [N, K] (fp32).
 cudaError_t split6_weights(const float* w, int N, int K, void* out, cudaStream_t st);
 GemmASplit split3_a_map(int K);
@@ -165,20 +170,17 @@ cudaError_t rmsnorm_f32_to_bf16(const float* x, const float* gain, void* out, in
                                 const int* row_count, int d, float eps, cudaStream_t st);
 cudaError_t rmsnorm_f32_to_f32(const float* x, const float* gain, float* out, int rows_cap,
                                const int* row_count, int d, float eps, cudaStream_t st);
-cudaError_t layernorm_f32(const float* x, int ldx, const float* gain, const float* bias, float* out_f32,
-                          void* out_bf16, int ldo, int rows, int d, float eps, float scale,
-                          cudaStream_t st);
+cudaError_t layernorm_bf16(const float* x, const float* gain, const float* bias, void* out, int rows, int d, float eps,
+                           cudaStream_t st);
 // Zeroes rows [T, T + nrows) (below rows_cap) of a row-major buffer, T = *row_count.
 cudaError_t zero_rows_after(void* buf, size_t row_bytes, const int* row_count, int rows_cap, int nrows,
                             cudaStream_t st);
 cudaError_t bf16_to_f32(const void* x, float* out, int rows_cap, const int* row_count, int d,
                         cudaStream_t st);
+// Encoder input rows into R, the first block's LN1 of them into A (bf16) and the sequences' offsets into cu.
 cudaError_t assemble_encoder_input(const BatchDesc& bd, const void* X, const float* P, int D,
-                                   const float* ln_g, const float* ln_b, float eps, float g_text,
-                                   float* R, int rows, cudaStream_t st);
-cudaError_t gather_memory(const BatchDesc& bd, const float* R, const float* H, const float* s_stop,
-                          const float* s_start, float* Mall, int D, cudaStream_t st);
-cudaError_t write_enc_cu(const BatchDesc& bd, int* cu, cudaStream_t st);
+                                   const float* ln_g, const float* ln_b, const float* ln1_g, const float* ln1_b,
+                                   float eps, float g_text, float* R, void* A, int rows, int* cu, cudaStream_t st);
 
 // ------------------------------------------------------------- key / value cache and decode
 // Cache layout: layer block [2][B][S_cap][Hkv * dh] bf16 (K then V).

@@ -31,24 +31,6 @@ SP_DEVINL void split3(float x, __nv_bfloat16& p0, __nv_bfloat16& p1, __nv_bfloat
   p2 = __float2bfloat16_rn(r2);
 }
 
-// out[r, s*K + k] = part s of x[r, k], s = 0, 1, 2 (4 elements per thread).
-__global__ void split3_kernel(const float* __restrict__ x, int ldx, int rows, int K, __nv_bfloat16* __restrict__ out) {
-  const int q = K >> 2;
-  const long long n = (long long)rows * q;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(i / q), k = (int)(i - (long long)r * q) * 4;
-    const float4 v = *reinterpret_cast<const float4*>(x + (size_t)r * ldx + k);
-    __nv_bfloat16 a[3][4];
-    split3(v.x, a[0][0], a[1][0], a[2][0]);
-    split3(v.y, a[0][1], a[1][1], a[2][1]);
-    split3(v.z, a[0][2], a[1][2], a[2][2]);
-    split3(v.w, a[0][3], a[1][3], a[2][3]);
-    __nv_bfloat16* o = out + (size_t)r * 3 * K + k;
-#pragma unroll
-    for (int s = 0; s < 3; ++s) *reinterpret_cast<uint2*>(o + (size_t)s * K) = *reinterpret_cast<const uint2*>(a[s]);
-  }
-}
-
 // out[n, s*K + k] = part pat[s] of w[n, k] for the six weight segments.
 __global__ void split6_weights_kernel(const float* __restrict__ w, int N, int K, __nv_bfloat16* __restrict__ out) {
   const long long n = (long long)N * K;
@@ -82,17 +64,6 @@ GemmASplit split3_a_map(int K) {
   s.seg = K;
   s.map = (0u << 0) | (0u << 4) | (1u << 8) | (0u << 12) | (1u << 16) | (2u << 20);
   return s;
-}
-
-cudaError_t split3_bf16(const float* x, int ldx, int rows, int K, void* out, cudaStream_t st) {
-  if (rows <= 0) return cudaSuccess;
-  if (K % 4 != 0 || ldx % 4 != 0) return cudaErrorInvalidValue;
-  const long long n = (long long)rows * (K / 4);
-  const int grid = (int)std::min<long long>((n + 255) / 256, (long long)device_sm_count() * 16);
-  prof_begin_launch(st);
-  split3_kernel<<<grid, 256, 0, st>>>(x, ldx, rows, K, reinterpret_cast<__nv_bfloat16*>(out));
-  prof_end_launch(st, SP_K_SGEMM, 0.0, (double)rows * K * (4.0 + 6.0));
-  return cudaGetLastError();
 }
 
 cudaError_t split6_weights(const float* w, int N, int K, void* out, cudaStream_t st) {

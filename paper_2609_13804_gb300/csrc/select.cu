@@ -249,6 +249,8 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int h = a.h, k_max = a.k_max, g = a.g;
   const int per = g + 1;
+  pdl_wait();
+  pdl_trigger();
 
   // episode geometry
   int lo = 0, hi = bd.B - 1;
@@ -1165,10 +1167,12 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
 // Algorithm 1 step 4: per image, the union of its episodes' selections in
 // native (ascending) order, -1 padded to k_cap.
 __global__ void __launch_bounds__(512)
-restore_kernel(const BatchDesc bd, const int* __restrict__ order, const int* __restrict__ ep_count,
+restore_kernel(const BatchDesc bd, const int* order, const int* ep_count,
                int k_max, int* __restrict__ idx, int k_cap, int* __restrict__ count, int* err) {
   extern __shared__ uint8_t flags[];
   __shared__ int wsum[32];
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.x, tid = threadIdx.x, NTR = blockDim.x;
   const int n_img = bd.vis_off[b + 1] - bd.vis_off[b];
   const int gs = bd.group_size > 0 ? bd.group_size : n_img;
@@ -1299,13 +1303,15 @@ cudaError_t select_launch(const BatchDesc& bd, int n_episodes, const SelectArgs&
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = L.total;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
   prof_begin_launch(st);
   r = cudaLaunchKernelEx(&cfg, kern, bd, a, n_loc, keys_in_smem ? 1 : 0, tm_cols);
   prof_end_launch(st, SP_K_SELECT, 0.0, 0.0);
@@ -1321,9 +1327,10 @@ cudaError_t restore_launch(const BatchDesc& bd, const int* order, const int* ep_
     if (r != cudaSuccess) return r;
   }
   prof_begin_launch(st);
-  restore_kernel<<<bd.B, 512, n_max, st>>>(bd, order, ep_count, k_max, idx, k_cap, count, err);
+  const cudaError_t r = launch_pdl(restore_kernel, dim3(bd.B), dim3(512), (size_t)n_max, st, bd, order, ep_count, k_max,
+                                   idx, k_cap, count, err);
   prof_end_launch(st, SP_K_RESTORE, 0.0, 0.0);
-  return cudaGetLastError();
+  return r;
 }
 
 }  // namespace sp
