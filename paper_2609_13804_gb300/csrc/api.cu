@@ -232,12 +232,16 @@ using namespace sp;
 struct sp_selector_s {
   sp_selector_cfg cfg;
   sp_selector_weights w;
-  // candidate precompute weights as six bf16 segments b0 b1 b0 b2 b1 b0 of
+  // candidate precompute weights as three fp16 segments b1 b2 b1 of the scaled rows (P1s, P2s), and Wcat1 also as
+  // six bf16 segments (P1w: grouped rounds, wide memories) of
   //   Wcat1 [2h, D]: rows W_in | Wq_p^T Wk_p / sqrt(h)
   //   Wcat2 [3h, h]: rows Wq_s / sqrt(h) | Wk_s | Wo_s Wv_s
-  void* P1s = nullptr;  // [2h, 6D]
-  void* P2s = nullptr;  // [3h, 6h]
-  GemmB P1, P2;
+  void* P1s = nullptr;  // [2h, 3D] (NULL: D > kSplit2MaxD)
+  void* P1w = nullptr;  // [2h, 6D]
+  void* P2s = nullptr;  // [3h, 3h]
+  float* P1i = nullptr;  // [2h] inverse scales
+  float* P2i = nullptr;  // [3h]
+  GemmB P1, P1w3, P2;
   GemmB Wp;
   // decoders of several layers: Wcat1 also holds, per layer before the last,
   // Wq_c^T Wk_c / sqrt(h) | Wo_c Wv_c; the runtime weights of layers >= 1
@@ -340,11 +344,15 @@ sp_status sp_selector_create(const sp_selector_cfg* cfg, const sp_selector_weigh
   s->pre_ln1_g = low ? low[0].ln1_g : w->ln1_g;
   s->pre_ln1_b = low ? low[0].ln1_b : w->ln1_b;
   const int r1 = 2 * nd;  // row blocks of h in Wcat1
+  const bool two = D <= kSplit2MaxD;
   float *Wcat1 = nullptr, *Wcat2 = nullptr;
   cudaError_t e = cudaMalloc(&Wcat1, (size_t)r1 * h * D * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&Wcat2, (size_t)3 * h * h * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&s->P1s, (size_t)r1 * h * 6 * D * sizeof(uint16_t));
-  if (e == cudaSuccess) e = cudaMalloc(&s->P2s, (size_t)3 * h * 6 * h * sizeof(uint16_t));
+  if (e == cudaSuccess && two) e = cudaMalloc(&s->P1s, (size_t)r1 * h * 3 * D * sizeof(uint16_t));
+  if (e == cudaSuccess) e = cudaMalloc(&s->P1w, (size_t)r1 * h * 6 * D * sizeof(uint16_t));
+  if (e == cudaSuccess) e = cudaMalloc(&s->P2s, (size_t)3 * h * 3 * h * sizeof(uint16_t));
+  if (e == cudaSuccess) e = cudaMalloc(&s->P1i, (size_t)r1 * h * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&s->P2i, (size_t)3 * h * sizeof(float));
   if (e == cudaSuccess && nd > 1) e = cudaMalloc(&s->Wf, (size_t)(nd - 1) * 3 * h * h * sizeof(float));
   if (e == cudaSuccess && nd > 1) e = cudaMalloc(&s->dec_dev, (size_t)nd * sizeof(DecLayerDev));
   const float rs = 1.0f / std::sqrt((float)h);
@@ -395,8 +403,9 @@ sp_status sp_selector_create(const sp_selector_cfg* cfg, const sp_selector_weigh
     }
   }
   if (e == cudaSuccess && nd > 1) e = cudaMemcpy(s->dec_dev, dd.data(), nd * sizeof(DecLayerDev), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = split6_weights(Wcat1, r1 * h, D, s->P1s, 0);
-  if (e == cudaSuccess) e = split6_weights(Wcat2, 3 * h, h, s->P2s, 0);
+  if (e == cudaSuccess && two) e = split_weights(Wcat1, r1 * h, D, 2, s->P1s, s->P1i, 0);
+  if (e == cudaSuccess) e = split_weights(Wcat1, r1 * h, D, 3, s->P1w, nullptr, 0);
+  if (e == cudaSuccess) e = split_weights(Wcat2, 3 * h, h, 2, s->P2s, s->P2i, 0);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (dI) cudaFree(dI);
   if (Wcat1) cudaFree(Wcat1);
@@ -406,7 +415,8 @@ sp_status sp_selector_create(const sp_selector_cfg* cfg, const sp_selector_weigh
     return cuda_fail(e, "sp_selector_create (fold)");
   }
   std::string msg;
-  bool ok = make_gemm_b(&s->P1, s->P1s, r1 * h, 6 * D, &msg) && make_gemm_b(&s->P2, s->P2s, 3 * h, 6 * h, &msg);
+  bool ok = (!two || make_gemm_b(&s->P1, s->P1s, r1 * h, 3 * D, &msg)) &&
+            make_gemm_b(&s->P1w3, s->P1w, r1 * h, 6 * D, &msg) && make_gemm_b(&s->P2, s->P2s, 3 * h, 3 * h, &msg);
   if (ok && c.n_enc_layers > 0) {
     ok = make_gemm_b(&s->Wp, w->W_p, D, c.D_text, &msg);
     for (int i = 0; ok && i < c.n_enc_layers; ++i) {
@@ -427,7 +437,10 @@ sp_status sp_selector_create(const sp_selector_cfg* cfg, const sp_selector_weigh
 void sp_selector_destroy(sp_selector* s) {
   if (!s) return;
   if (s->P1s) cudaFree(s->P1s);
+  if (s->P1w) cudaFree(s->P1w);
   if (s->P2s) cudaFree(s->P2s);
+  if (s->P1i) cudaFree(s->P1i);
+  if (s->P2i) cudaFree(s->P2i);
   if (s->Wf) cudaFree(s->Wf);
   if (s->dec_dev) cudaFree(s->dec_dev);
   delete s;
@@ -617,31 +630,42 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
     if (rs != SP_OK) return rs;
   }
   void* Asp = parts[14];
+  const int parts1 = s->P1s && in->g == 1 ? 2 : 3;  // (precompute.cu)
+  // the rows' inverse scales, behind the widest operand's two parts
+  float* Ainv = reinterpret_cast<float*>(static_cast<uint16_t*>(Asp) + (size_t)p.rows * 2 * std::max(D, h));
   SP_CUDA(memory_split(p.bd, blocks ? (float*)parts[1] : nullptr, in->H, blocks ? nullptr : in->X, s->w.s_stop,
-                       s->w.s_start, Asp, out->memory, D, st),
+                       s->w.s_start, Asp, parts1 == 2 ? Ainv : nullptr, out->memory, D, st),
           "memory");
   float* ZK = (float*)parts[8];
   float* QKVs = (float*)parts[10];
   // candidate precompute (fp32): [z | KT] = M [W_in; Wq_p^T Wk_p / sqrt h]^T, x = LN1(z),
   // [QS | KS | VT] = x [Wq_s / sqrt h; Wk_s; Wo_s Wv_s]^T
-  // (fp32-accurate products on the bf16 tensor cores: three-way operand split)
+  // (fp32-accurate products on the fp16 tensor cores: two-way operand split)
   {
     std::string msg;
     CUtensorMap t1, t2;
-    if (!encode_tmap_bf16(&t1, Asp, p.rows, 3 * D, 128, &msg) || !encode_tmap_bf16(&t2, Asp, p.rows, 3 * h, 128, &msg))
+    if (!encode_tmap_bf16(&t1, Asp, p.rows, parts1 * D, 128, &msg) || !encode_tmap_bf16(&t2, Asp, p.rows, 2 * h, 128, &msg))
       return fail(SP_ERR_CUDA, "%s", msg.c_str());
     GemmEpi e1;
     e1.kind = EPI_F32;
     e1.out = ZK;
     e1.ldo = 2 * s->n_dec * h;
-    const GemmASplit a1 = split3_a_map(D), a2 = split3_a_map(h);
-    SP_CUDA(gemm_bf16(t1, p.rows, nullptr, s->P1, 2 * s->n_dec * h, e1, err, st, nullptr, &a1), "precompute 1");
-    SP_CUDA(layernorm_split(ZK, 2 * s->n_dec * h, s->pre_ln1_g, s->pre_ln1_b, Asp, p.rows, h, s->cfg.ln_eps, st),
+    if (parts1 == 2) {
+      e1.row_scale = Ainv;
+      e1.col_scale = s->P1i;
+    }
+    const GemmASplit a1 = split_a_map(D, parts1), a2 = split_a_map(h, 2);
+    SP_CUDA(gemm_bf16(t1, p.rows, nullptr, parts1 == 2 ? s->P1 : s->P1w3, 2 * s->n_dec * h, e1, err, st, nullptr, &a1),
+            "precompute 1");
+    SP_CUDA(layernorm_split(ZK, 2 * s->n_dec * h, s->pre_ln1_g, s->pre_ln1_b, Asp, Ainv, p.rows, h, s->cfg.ln_eps,
+                            st),
             "ln1");
     GemmEpi e2;
     e2.kind = EPI_F32;
     e2.out = QKVs;
     e2.ldo = 3 * h;
+    e2.row_scale = Ainv;
+    e2.col_scale = s->P2i;
     SP_CUDA(gemm_bf16(t2, p.rows, nullptr, s->P2, 3 * h, e2, err, st, nullptr, &a2), "precompute 2");
   }
 

@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include "stepprune.h"
@@ -50,6 +51,34 @@ SP_DEVINL uint32_t pack_bf16x2(float lo, float hi) {
 SP_DEVINL float2 unpack_bf16x2(uint32_t u) {
   __nv_bfloat162 v = *reinterpret_cast<__nv_bfloat162*>(&u);
   return __bfloat1622float2(v);
+}
+
+// The power of two that brings m (the largest magnitude of a row) into
+// [2^14, 2^15), and its inverse; 1 for zero, infinity and NaN.
+SP_DEVINL float split_scale(float m, float* inv) {
+  const int eb = (int)((__float_as_uint(m) >> 23) & 255u);  // exponent + 127
+  const int sb = (eb == 0 || eb == 255) ? 127 : min(268 - eb, 253);
+  *inv = __uint_as_float((uint32_t)(254 - sb) << 23);
+  return __uint_as_float((uint32_t)sb << 23);
+}
+
+SP_DEVINL float max_abs4(const float4& v) {
+  return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+}
+
+// Two fp16 parts of four floats times sc (split_scale of their row): x sc =
+// a + b up to 2^-23 |x sc|, or 2^-25 where b is subnormal.
+SP_DEVINL void split2_f16(const float4& v, float sc, uint2& a, uint2& b) {
+  const float x[4] = {v.x * sc, v.y * sc, v.z * sc, v.w * sc};
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const __half p = __float2half_rn(x[c]);
+    h[c] = __half_as_ushort(p);
+    l[c] = __half_as_ushort(__float2half_rn(x[c] - __half2float(p)));
+  }
+  a = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+  b = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
 }
 
 SP_DEVINL float gelu_erf(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
@@ -574,6 +603,11 @@ SP_DEVINL uint64_t umma_desc_sw128_mn(uint32_t smem_addr, uint32_t lbo) {
 __host__ __device__ constexpr uint32_t umma_idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
+}
+
+// The same with A and B fp16 (formats 0).
+__host__ __device__ constexpr uint32_t umma_idesc_f16_f32(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 }  // namespace sp

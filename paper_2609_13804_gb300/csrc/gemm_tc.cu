@@ -300,10 +300,23 @@ SP_DEVINL void epilogue_tma(const GemmEpi& e, const CUtensorMap* tmO, uint32_t t
                             bool live, int nb, uint8_t* boxes, int& nbox, const Fix& fx, int* err) {
   float v[32];
   if (EPI == EPI_F32 || EPI == EPI_F32_ACC) {
+    const bool scaled = EPI == EPI_F32 && e.row_scale != nullptr;
+    const float rs = scaled && live ? __ldg(e.row_scale + row0 + lane) : 0.f;
 #pragma unroll 1
     for (int c = 0; c < BN / 32; ++c) {
       tmem_ld_32x32b_x32(taddr + c * 32, v);
       fix_add_waited(fx, c * 32, v);
+      if (scaled) {
+        const float4* cs = reinterpret_cast<const float4*>(e.col_scale + nb * BN + c * 32);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float4 w = __ldg(cs + q);
+          v[4 * q] *= rs * w.x;
+          v[4 * q + 1] *= rs * w.y;
+          v[4 * q + 2] *= rs * w.z;
+          v[4 * q + 3] *= rs * w.w;
+        }
+      }
       if (!live) zero32(v);
       if (lane == 0) bulk_wait_read<1>();
       __syncwarp();
@@ -619,7 +632,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (one thread)
     if (lane == 0) {
-      constexpr uint32_t IDESC = umma_idesc_bf16_f32(BM, BN);
+      const uint32_t IDESC = EPI == EPI_F32 && args.e.row_scale ? umma_idesc_f16_f32(BM, BN) : umma_idesc_bf16_f32(BM, BN);
       int s = 0;
       uint32_t ph = 0;
       int it = 0;
@@ -941,7 +954,8 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (one thread of the even CTA)
     if (leader && lane == 0) {
-      constexpr uint32_t IDESC = umma_idesc_bf16_f32(2 * BM, BN);
+      const uint32_t IDESC =
+          EPI == EPI_F32 && args.e.row_scale ? umma_idesc_f16_f32(2 * BM, BN) : umma_idesc_bf16_f32(2 * BM, BN);
       int s = 0;
       uint32_t ph = 0;
       int it = 0;
@@ -1478,6 +1492,7 @@ cudaError_t gemm_bf16(const CUtensorMap& A, int M_cap, const int* M_dev, const G
                       const GemmEpi& e, int* err, cudaStream_t st, const GemmScratch* sk,
                       const GemmASplit* as, const CUtensorMap* A16, const int* a_rows) {
   if (M_cap <= 0) return cudaSuccess;
+  if (e.row_scale && (e.kind != EPI_F32 || sk || !e.col_scale)) return cudaErrorInvalidValue;
   const int sms = device_sm_count();
   if (a_rows) A16 = nullptr;  // gathered A rows: not the weight-streaming form (M <= 32 rows)
   // Weight streaming for M <= 32 rows (generation steps): the weights are the

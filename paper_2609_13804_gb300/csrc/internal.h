@@ -84,6 +84,9 @@ struct GemmEpi {
   int max_pos = 0;
   int head_dim = 0;
   int rope_cols = 0;
+  // EPI_F32 without scratch: A and B are fp16, out = acc * row_scale[row] * col_scale[column] (NULL: bf16, unscaled)
+  const float* row_scale = nullptr;
+  const float* col_scale = nullptr;  // 16-byte aligned
   int up_off = 0;                    // EPI_SWIGLU_BF16: row of B where the 'up' half starts
 };
 
@@ -151,16 +154,20 @@ cudaError_t gemm_bf16(const CUtensorMap& A, int M_cap, const int* M_dev, const G
                       const CUtensorMap* A16 = nullptr, const int* a_rows = nullptr);
 
 // ------------------------------------------------------------- candidate precompute
-// The candidate memory [visual rows of H, of X (bf16) or of the encoder's R; s_stop; s_start] as its three bf16
-// parts, out [rows, 3D]; memory (may be NULL) receives the visual rows in fp32.
+// Widest candidate memory whose first precompute product takes two fp16 parts with g = 1 (precompute.cu).
+constexpr int kSplit2MaxD = 1536;
+// The candidate memory [visual rows of H, of X (bf16) or of the encoder's R; s_stop; s_start] as its two scaled
+// fp16 parts, out [rows, 2D], and their inverse scales inv [rows], or (inv NULL) as its three bf16 parts, out
+// [rows, 3D]; memory (may be NULL) receives the visual rows in fp32.
 cudaError_t memory_split(const BatchDesc& bd, const float* R, const float* H, const void* X, const float* s_stop,
-                         const float* s_start, void* out, float* memory, int D, cudaStream_t st);
-// LN of fp32 rows (d <= 1,024, ldx apart) as their three bf16 parts, out [rows, 3d].
-cudaError_t layernorm_split(const float* x, int ldx, const float* gain, const float* bias, void* out, int rows, int d,
-                            float eps, cudaStream_t st);
-// out [N, 6K] bf16 = the weight segments b0 b1 b0 b2 b1 b0 of w [N, K] (fp32).
-cudaError_t split6_weights(const float* w, int N, int K, void* out, cudaStream_t st);
-GemmASplit split3_a_map(int K);
+                         const float* s_start, void* out, float* inv, float* memory, int D, cudaStream_t st);
+// LN of fp32 rows (d <= 1,024, ldx apart) as their two scaled fp16 parts, out [rows, 2d], and inverse scales.
+cudaError_t layernorm_split(const float* x, int ldx, const float* gain, const float* bias, void* out, float* inv,
+                            int rows, int d, float eps, cudaStream_t st);
+// The weight segments of w [N, K] (fp32, K a multiple of 4): two parts, out [N, 3K] fp16 and inverse scales inv [N],
+// or three, out [N, 6K] bf16.
+cudaError_t split_weights(const float* w, int N, int K, int parts, void* out, float* inv, cudaStream_t st);
+GemmASplit split_a_map(int K, int parts);
 cudaError_t fold_matmul(const float* A, long sai, long sak, const float* B, long sbk, long sbj,
                         float* C, int ldc, int I, int J, int K, float scale, cudaStream_t st);
 

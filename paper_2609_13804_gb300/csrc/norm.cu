@@ -327,26 +327,19 @@ assemble_wide_kernel(const BatchDesc bd, const __nv_bfloat16* X, const float* P,
   }
 }
 
-// Three bf16 parts of four floats: x = p0 + p1 + p2 (+ about 2^-24 x).
-SP_DEVINL void split3(const float4& v, uint2 (&o)[3]) {
-  float r[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    o[s] = make_uint2(pack_bf16x2(r[0], r[1]), pack_bf16x2(r[2], r[3]));
-    const float2 lo = unpack_bf16x2(o[s].x), hi = unpack_bf16x2(o[s].y);
-    r[0] -= lo.x; r[1] -= lo.y; r[2] -= hi.x; r[3] -= hi.y;
-  }
-}
-
 // Candidate memory rows [every image's visual rows; s_stop; s_start] (row
 // sources: the encoder's residual R, the given memory H, or the visual tokens X
-// themselves) as the split operand of the precompute GEMM, [rows, 3D] bf16
-// (parts p0 | p1 | p2), and optionally the visual rows to `memory` (fp32).  One
-// pass in place of a gathered copy that a split pass re-read: HBM-bound, a warp
-// per row with up to eight 16-byte loads per lane in flight.
+// themselves) as the split operand of the precompute GEMM: [rows, 2D] fp16
+// (parts a1 | a2 of the scaled row) with the inverse scales, or [rows, 3D] bf16
+// (PARTS = 3); optionally the visual rows go to `memory` (fp32).  HBM-bound, a
+// warp per row.  NV > 0: all of the row's 16-byte loads in flight, the row held
+// in registers (NV float4 per lane) between the search for its largest element
+// and the split; NV = 0 (rows wider than that): read twice for PARTS = 2.
+template <int NV, int PARTS>
 __global__ void __launch_bounds__(NT)
 memory_split_kernel(const BatchDesc bd, const float* R, const float* H, const uint2* X, const float* s_stop,
-                    const float* s_start, uint2* out, float* memory, int n4, int rows, int vec_ends, int vec_mem) {
+                    const float* s_start, uint2* out, float* inv, float* memory, int n4, int rows, int vec_ends,
+                    int vec_mem) {
   pdl_wait();
   pdl_trigger();
   const int r = blockIdx.x * (NT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -366,50 +359,68 @@ memory_split_kernel(const BatchDesc bd, const float* R, const float* H, const ui
     const int b = find_image(bd.vis_off, bd.B, r);
     src = R + (size_t)(r + bd.txt_off[b]) * 4 * n4;
   }
-  uint2* o = out + (size_t)r * 3 * n4;
+  uint2* o = out + (size_t)r * PARTS * n4;
   float* mem = memory && r < nvis ? memory + (size_t)r * 4 * n4 : nullptr;
-  constexpr int U = 8;
-  for (int i0 = lane; i0 < n4; i0 += 32 * U) {
-    float4 v[U];
+  auto load = [&](int i) {
+    if (xs) {
+      const uint2 w = xs[i];
+      const float2 lo = unpack_bf16x2(w.x), hi = unpack_bf16x2(w.y);
+      return make_float4(lo.x, lo.y, hi.x, hi.y);
+    }
+    if (vec) return reinterpret_cast<const float4*>(src)[i];
+    return make_float4(src[4 * i], src[4 * i + 1], src[4 * i + 2], src[4 * i + 3]);
+  };
+  auto put = [&](int i, const float4& v, float sc) {
+    if constexpr (PARTS == 2) {
+      split2_f16(v, sc, o[i], o[n4 + i]);
+    } else {
+      float x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = i0 + 32 * u;
-      if (i >= n4) continue;
-      if (xs) {
-        const uint2 w = xs[i];
-        const float2 lo = unpack_bf16x2(w.x), hi = unpack_bf16x2(w.y);
-        v[u] = make_float4(lo.x, lo.y, hi.x, hi.y);
-      } else if (vec) {
-        v[u] = reinterpret_cast<const float4*>(src)[i];
+      for (int s = 0; s < 3; ++s) {
+        const uint2 u = make_uint2(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]));
+        const float2 lo = unpack_bf16x2(u.x), hi = unpack_bf16x2(u.y);
+        x[0] -= lo.x; x[1] -= lo.y; x[2] -= hi.x; x[3] -= hi.y;
+        o[s * n4 + i] = u;
+      }
+    }
+    if (mem) {
+      if (vec_mem) {
+        reinterpret_cast<float4*>(mem)[i] = v;
       } else {
-        v[u] = make_float4(src[4 * i], src[4 * i + 1], src[4 * i + 2], src[4 * i + 3]);
+        mem[4 * i] = v.x; mem[4 * i + 1] = v.y; mem[4 * i + 2] = v.z; mem[4 * i + 3] = v.w;
       }
     }
+  };
+  float m = 0.f, iv;
+  if constexpr (NV > 0) {
+    float4 v[NV];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = i0 + 32 * u;
-      if (i >= n4) continue;
-      uint2 p[3];
-      split3(v[u], p);
+    for (int k = 0; k < NV; ++k)
+      if (lane + 32 * k < n4) v[k] = load(lane + 32 * k);
 #pragma unroll
-      for (int s = 0; s < 3; ++s) o[(size_t)s * n4 + i] = p[s];
-      if (mem) {
-        if (vec_mem) {
-          reinterpret_cast<float4*>(mem)[i] = v[u];
-        } else {
-          mem[4 * i] = v[u].x; mem[4 * i + 1] = v[u].y; mem[4 * i + 2] = v[u].z; mem[4 * i + 3] = v[u].w;
-        }
-      }
-    }
+    for (int k = 0; k < NV; ++k)
+      if (lane + 32 * k < n4) m = fmaxf(m, max_abs4(v[k]));
+    const float sc = split_scale(warp_max(m), &iv);
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      if (lane + 32 * k < n4) put(lane + 32 * k, v[k], sc);
+  } else {
+#pragma unroll 4
+    for (int i = PARTS == 2 ? lane : n4; i < n4; i += 32) m = fmaxf(m, max_abs4(load(i)));
+    const float sc = split_scale(warp_max(m), &iv);
+#pragma unroll 4
+    for (int i = lane; i < n4; i += 32) put(i, load(i), sc);
   }
+  if (PARTS == 2 && lane == 0) inv[r] = iv;
 }
 
 // LN1 of the decoder tokens (rows of h floats, ldx apart) as the split operand of
-// the second precompute GEMM, [rows, 3h] bf16; a warp per row (h <= 1,024).
+// the second precompute GEMM, [rows, 2h] fp16, and its inverse scales; a warp per
+// row (h <= 1,024).
 template <int NV>
 __global__ void __launch_bounds__(NT)
 layernorm_split_kernel(const float* x, int ldx, const float* __restrict__ gain,
-                       const float* __restrict__ bias, int vec, uint2* out, int rows, int n4, float eps) {
+                       const float* __restrict__ bias, int vec, uint2* out, float* inv, int rows, int n4, float eps) {
   pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x & 31;
@@ -421,14 +432,16 @@ layernorm_split_kernel(const float* x, int ldx, const float* __restrict__ gain,
   for (int k = 0; k < NV; ++k)
     if (lane + 32 * k < n4) v[k] = xr[lane + 32 * k];
   row_layernorm<NV>(v, lane, n4, gain, bias, vec != 0, eps);
+  float m = 0.f, iv;
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    if (lane + 32 * k >= n4) continue;
-    uint2 p[3];
-    split3(v[k], p);
+  for (int k = 0; k < NV; ++k)
+    if (lane + 32 * k < n4) m = fmaxf(m, max_abs4(v[k]));
+  const float sc = split_scale(warp_max(m), &iv);
+  if (lane == 0) inv[row] = iv;
 #pragma unroll
-    for (int s = 0; s < 3; ++s) out[((size_t)row * 3 + s) * n4 + lane + 32 * k] = p[s];
-  }
+  for (int k = 0; k < NV; ++k)
+    if (lane + 32 * k < n4)
+      split2_f16(v[k], sc, out[(size_t)row * 2 * n4 + lane + 32 * k], out[((size_t)row * 2 + 1) * n4 + lane + 32 * k]);
 }
 
 }  // namespace
@@ -489,16 +502,16 @@ cudaError_t layernorm_bf16(const float* x, const float* gain, const float* bias,
   return r;
 }
 
-cudaError_t layernorm_split(const float* x, int ldx, const float* gain, const float* bias, void* out, int rows, int d,
-                            float eps, cudaStream_t st) {
+cudaError_t layernorm_split(const float* x, int ldx, const float* gain, const float* bias, void* out, float* inv,
+                            int rows, int d, float eps, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
   if (d > 1024 || d % 4 != 0 || ldx % 4 != 0) return cudaErrorInvalidValue;
   prof_begin_launch(st);
   const cudaError_t r = with_row_form(d, [&](auto nv) {
     return launch_pdl(layernorm_split_kernel<decltype(nv)::value>, dim3(row_blocks(rows)), dim3(NT), 0, st, x, ldx,
-                      gain, bias, aligned16(gain, bias) ? 1 : 0, static_cast<uint2*>(out), rows, d / 4, eps);
+                      gain, bias, aligned16(gain, bias) ? 1 : 0, static_cast<uint2*>(out), inv, rows, d / 4, eps);
   });
-  prof_end_launch(st, SP_K_NORM, 0.0, 10.0 * rows * (double)d);
+  prof_end_launch(st, SP_K_NORM, 0.0, 8.0 * rows * (double)d);
   return r;
 }
 
@@ -547,13 +560,17 @@ cudaError_t assemble_encoder_input(const BatchDesc& bd, const void* X, const flo
 }
 
 cudaError_t memory_split(const BatchDesc& bd, const float* R, const float* H, const void* X, const float* s_stop,
-                         const float* s_start, void* out, float* memory, int D, cudaStream_t st) {
+                         const float* s_start, void* out, float* inv, float* memory, int D, cudaStream_t st) {
   const int rows = bd.vis_off[bd.B] + 2;
   prof_begin_launch(st);
-  const cudaError_t r = launch_pdl(memory_split_kernel, dim3(row_blocks(rows)), dim3(NT), 0, st, bd, R, H,
-                                   static_cast<const uint2*>(X), s_stop, s_start, static_cast<uint2*>(out), memory,
-                                   D / 4, rows, aligned16(s_stop, s_start) ? 1 : 0, aligned16(memory, nullptr) ? 1 : 0);
-  prof_end_launch(st, SP_K_SGEMM, 0.0, (memory ? 14.0 : 10.0) * rows * (double)D);
+  auto go = [&](auto nv) {
+    constexpr int NV = decltype(nv)::value;
+    return launch_pdl(inv ? memory_split_kernel<NV, 2> : memory_split_kernel<NV, 3>, dim3(row_blocks(rows)), dim3(NT), 0, st, bd, R, H,
+                      static_cast<const uint2*>(X), s_stop, s_start, static_cast<uint2*>(out), inv, memory, D / 4, rows,
+                      aligned16(s_stop, s_start) ? 1 : 0, aligned16(memory, nullptr) ? 1 : 0);
+  };
+  const cudaError_t r = D <= kRowFormMax ? with_row_form(D, go) : go(std::integral_constant<int, 0>{});
+  prof_end_launch(st, SP_K_SGEMM, 0.0, (memory ? 12.0 : 8.0) * rows * (double)D);
   return r;
 }
 
