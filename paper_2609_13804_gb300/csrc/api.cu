@@ -452,7 +452,45 @@ struct SelPlan {
   BatchDesc bd;
   int E = 0, nvis = 0, ntxt = 0, T_enc = 0, max_enc = 0, rows = 0, k_max = 0;
   bool encoder = false;
+  // the table-driven selection (gram.cu): its plan, and its cluster size (0: the general kernel)
+  GramArgs gram = {};
+  int n_max = 0, gram_C = 0;
 };
+
+size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* out, Carve& cv, void** parts);
+
+// Whether the selection goes through per-episode tables.  They cost kGramFixedUs
+// and 30 h (n + 2)^2 tensor operations per episode (16 x 576 candidates, h = 512:
+// 155 us with their operands, 0.53e9 a microsecond; one of 576, h = 256: 23 us)
+// and save kGramRoundUs of every round (16 x 576: 4.9 -> 2.5 us; training 6.8 ->
+// 2.6; one image 5.6 -> 2.1); the rounds are bounded by the cap (a STOP can end
+// them early, which only the device knows).
+constexpr double kGramFixedUs = 15.0;
+constexpr double kGramOpsPerUs = 0.55e9;
+constexpr double kGramRoundUs = 2.5;
+
+void plan_gram(const sp_selector* s, const sp_select_in* in, SelPlan* p) {
+  const int h = s->cfg.h;
+  if (s->n_dec != 1 || (h != 128 && h != 256 && h != 512 && h != 1024)) return;
+  double ops = 0.0;
+  for (int b = 0; b < in->B; ++b) {
+    const int n = in->n_vis[b], gs = in->group_size > 0 ? in->group_size : n;
+    p->n_max = std::max(p->n_max, std::min(gs, n));
+    ops += 30.0 * h * ((double)(n / gs) * (gs + 2.0) * (gs + 2.0) + (n % gs + 2.0) * (n % gs + 2.0));
+  }
+  const int rounds = (std::min(in->k_max, p->n_max) + in->g - 1) / in->g;
+  if (kGramFixedUs + ops / kGramOpsPerUs > kGramRoundUs * rounds) return;
+  const int C = select_gram_cluster(p->n_max, in->k_max, in->g);
+  if (C == 0) return;
+  gram_layout(p->E, p->nvis, p->n_max, h, &p->gram);
+  // A batch that the allocation-free entry point takes runs the same way with
+  // a caller's workspace: tables only if they fit its scratch too.
+  Carve base(nullptr), full(nullptr);
+  const size_t b0 = select_ws(s, *p, nullptr, base, nullptr) + 256;
+  p->gram_C = C;
+  const size_t b1 = select_ws(s, *p, nullptr, full, nullptr) + 256;
+  if (b0 <= SP_SELECT_NOALLOC_SCRATCH_BYTES && b1 > SP_SELECT_NOALLOC_SCRATCH_BYTES) p->gram_C = 0;
+}
 
 sp_status plan_select(const sp_selector* s, const sp_select_in* in, SelPlan* p) {
   if (!s || !in) return fail(SP_ERR_INVALID_ARG, "sp_select: NULL selector or input");
@@ -470,6 +508,7 @@ sp_status plan_select(const sp_selector* s, const sp_select_in* in, SelPlan* p) 
   p->T_enc = p->nvis + p->ntxt;
   p->max_enc = 0;
   for (int b = 0; b < in->B; ++b) p->max_enc = std::max(p->max_enc, in->n_vis[b] + in->n_txt[b]);
+  plan_gram(s, in, p);
   return SP_OK;
 }
 
@@ -492,20 +531,31 @@ size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* ou
   } else if (p.encoder) {
     R = cv.take<float>((size_t)p.T_enc * D);
   }
-  // (unused: the size that callers' workspaces and the allocation-free entry point's limit are checked
-  // against stays what it was when the memory and its LN1 were stored in fp32)
-  cv.take<float>((size_t)p.rows * D);
-  ZK = cv.take<float>((size_t)p.rows * 2 * s->n_dec * h);
-  cv.take<float>((size_t)p.rows * h);  // (unused, as above)
-  QKVs = cv.take<float>((size_t)p.rows * 3 * h);
+  // (the first two are unused by the general kernel: the size that callers' workspaces and the
+  // allocation-free entry point's limit are checked against stays what it was when the memory and its LN1
+  // were stored in fp32; the tables' operands take the place of all three after the precompute)
+  void* op = cv.take<float>((size_t)p.rows * D);
+  const size_t op0 = cv.off - (size_t)p.rows * D * sizeof(float);
+  cv.take<float>((size_t)p.rows * h);
   void* Asp = cv.take<uint16_t>((size_t)p.rows * 3 * std::max(D, h));  // split operand of the precompute GEMMs
+  if (p.gram_C) {
+    const size_t need = (size_t)p.gram.rows * (20 * h + 7 * sizeof(float));
+    if (cv.off - op0 < need) cv.off = op0 + need;
+  }
+  ZK = cv.take<float>((size_t)p.rows * 2 * s->n_dec * h);
+  const size_t tab0 = cv.off - (size_t)p.rows * 2 * s->n_dec * h * sizeof(float);
+  QKVs = cv.take<float>((size_t)p.rows * 3 * h);
+  if (p.gram_C) {  // the tables take the place of the precomputed rows once their operands are made
+    const size_t need = (size_t)p.E * p.gram.ep_stride * sizeof(float);
+    if (cv.off - tab0 < need) cv.off = tab0 + need;
+  }
   int* order = (out && out->order) ? nullptr : cv.take<int>((size_t)p.E * SP_MAX_KMAX);
   int* epc = (out && out->ep_count) ? nullptr : cv.take<int>((size_t)p.E);
   // self-attention rows of decoder layers >= 1, per episode and history position
   float* dcache = s->n_dec > 1 ? cv.take<float>((size_t)p.E * (s->n_dec - 1) * (p.k_max + 1) * 2 * h) : nullptr;
   if (parts) {
     parts[0] = P; parts[1] = R; parts[2] = Abf; parts[3] = QKV; parts[4] = O; parts[5] = F1;
-    parts[6] = enc_cu; parts[7] = nullptr; parts[8] = ZK; parts[9] = nullptr; parts[10] = QKVs;
+    parts[6] = enc_cu; parts[7] = op; parts[8] = ZK; parts[9] = nullptr; parts[10] = QKVs;
     parts[11] = order; parts[12] = epc; parts[13] = gsk; parts[14] = Asp; parts[15] = dcache;
   }
   return cv.off;
@@ -614,7 +664,12 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
   if (out->k_cap < need_cap) return fail(SP_ERR_SHAPE, "sp_select: k_cap %d < largest possible count %d", out->k_cap, need_cap);
   Carve cv(ws);
   void* parts[16];
-  const size_t need = select_ws(s, p, out, cv, parts) + 256;
+  size_t need = select_ws(s, p, out, cv, parts) + 256;
+  if (ws && ws_bytes < need && p.gram_C) {  // without room for the tables: the general kernel
+    p.gram_C = 0;
+    cv = Carve(ws);
+    need = select_ws(s, p, out, cv, parts) + 256;
+  }
   if (!ws || ws_bytes < need) return fail(SP_ERR_WORKSPACE, "sp_select: workspace %zu < %zu bytes", ws_bytes, need);
   if (!al16(ws)) return fail(SP_ERR_ALIGN, "sp_select: workspace must be 16-byte aligned");
   int* err = out->err;
@@ -694,10 +749,29 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
   a.KC = ZK + 2 * h;
   a.dcache = static_cast<float*>(parts[15]);
   a.dcache_ep = (size_t)(s->n_dec - 1) * (in->k_max + 1) * 2 * h;
-  bool keys_smem = true;
-  size_t smem = 0;
-  const int C = select_cluster_size(p.bd, h, in->k_max, &keys_smem, &smem, s->n_dec > 1);
-  SP_CUDA(select_launch(p.bd, p.E, a, C, keys_smem, smem, st), "selection");
+  if (p.gram_C) {
+    GramArgs ga = p.gram;
+    ga.Z = a.Z; ga.ldz = a.ldz;
+    ga.KT = a.KT; ga.ldkt = a.ldkt;
+    ga.QS = a.QS; ga.ldqs = a.ldqs;
+    ga.KS = a.KS; ga.ldks = a.ldks;
+    ga.VT = a.VT; ga.ldvt = a.ldvt;
+    ga.ln2_g = a.ln2_g; ga.ln2_b = a.ln2_b;
+    ga.stop_row = a.stop_row; ga.start_row = a.start_row;
+    ga.op = parts[7];
+    ga.inv = reinterpret_cast<float*>(static_cast<char*>(parts[7]) + (size_t)ga.rows * 20 * h);
+    ga.dj = ga.inv + (size_t)5 * ga.rows;
+    ga.zz = ga.dj + ga.rows;
+    ga.table = ZK;
+    ga.err = err;
+    SP_CUDA(gram_launch(p.bd, ga, st), "selection tables");
+    SP_CUDA(select_gram_launch(p.bd, p.E, a, ga, p.n_max, p.gram_C, st), "selection");
+  } else {
+    bool keys_smem = true;
+    size_t smem = 0;
+    const int C = select_cluster_size(p.bd, h, in->k_max, &keys_smem, &smem, s->n_dec > 1);
+    SP_CUDA(select_launch(p.bd, p.E, a, C, keys_smem, smem, st), "selection");
+  }
   SP_CUDA(restore_launch(p.bd, a.order, a.ep_count, in->k_max, out->idx, out->k_cap, out->count, err, st), "restore");
   return SP_OK;
 }

@@ -523,6 +523,13 @@ SP_DEVINL bool mbar_wait_cluster_warp(uint64_t* bar, uint32_t parity, int* err) 
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
+// Stores one word into a CTA of the cluster and counts its 4 bytes on that CTA's mbarrier
+// (both cluster shared-memory addresses).
+SP_DEVINL void st_async_u32(uint32_t cluster_addr, uint32_t v, uint32_t mbar_cluster_addr) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];"
+               ::"r"(cluster_addr), "r"(v), "r"(mbar_cluster_addr) : "memory");
+}
+
 // 2-D tiled TMA load into this CTA's shared memory whose completion is counted
 // on an mbarrier that may live in the peer CTA of the pair (cluster address).
 SP_DEVINL void tma_load_2d_pair(void* smem_dst, const void* tmap, uint32_t mbar_cluster_addr, int x, int y) {

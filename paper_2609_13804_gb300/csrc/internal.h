@@ -253,6 +253,34 @@ struct SelectArgs {
   size_t dcache_ep;         // floats per episode: (n_dec - 1) (k_max + 1) 2h
 };
 
+// Inner-product tables of the precomputed rows (gram.cu) and the selection that
+// reads them (select_gram.cu).
+struct GramArgs {
+  int E, rows, h;          // episodes, operand rows (every episode: candidates, STOP, START)
+  int ld;                  // columns of a table row (n_max + 2, a multiple of 4)
+  size_t ep_stride;        // floats per episode: (n_max + 2) rows of five table rows G | Gz | S | VV | ZV
+  int mt, nt, n_tile;      // row / column tiles of a table
+  const float* Z;  int ldz;
+  const float* KT; int ldkt;
+  const float* QS; int ldqs;
+  const float* KS; int ldks;
+  const float* VT; int ldvt;
+  const float* ln2_g; const float* ln2_b;
+  int stop_row, start_row;
+  void* op;                // [5][rows][2h] fp16: two parts of KTg, KS, vc, zc, QS
+  float* inv;              // [5][rows] inverse scales
+  float* dj;               // [rows] <kt, ln2 bias>
+  float* zz;               // [rows] |zc|^2
+  float* table;            // [E][ep_stride]
+  int* err;
+};
+void gram_layout(int E, int nvis, int n_max, int h, GramArgs* g);
+cudaError_t gram_launch(const BatchDesc& bd, const GramArgs& g, cudaStream_t st);
+// Cluster size of the table-driven selection, 0 where it does not take the episode sizes.
+int select_gram_cluster(int n_max, int k_max, int g);
+cudaError_t select_gram_launch(const BatchDesc& bd, int n_episodes, const SelectArgs& a, const GramArgs& g, int n_max,
+                               int C, cudaStream_t st);
+
 int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_smem, size_t* smem_bytes,
                         bool multi = false);
 cudaError_t select_launch(const BatchDesc& bd, int n_episodes, const SelectArgs& a,

@@ -30,10 +30,9 @@
 //   u = Z_last + sum_i softmax_i(<QS_last, KS_i>) VT_i.
 #include <cooperative_groups.h>
 
-#include <climits>
-
 #include "common.cuh"
 #include "internal.h"
+#include "select_common.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -99,17 +98,6 @@ __host__ __device__ inline SelSmem sel_layout(int h, int n_loc, int k_max, int C
   return L;
 }
 
-SP_DEVINL bool better(float v, int i, float bv, int bi) { return v > bv || (v == bv && i < bi); }
-
-SP_DEVINL void warp_best(float& v, int& i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, i, o);
-    if (better(ov, oi, v, i)) { v = ov; i = oi; }
-  }
-}
-
 // Sums of U independent per-lane values across the warp, reductions interleaved.
 template <int U>
 SP_DEVINL void warp_sum_n(float (&v)[U]) {
@@ -173,58 +161,6 @@ SP_DEVINL void top_insert(float (&tv)[GL], int (&ti)[GL], float v, int j, int ke
   if (better(v, j, tv[0], ti[0])) {
     tv[0] = v;
     ti[0] = j;
-  }
-}
-
-// Order-preserving 32-bit key of a float (larger float -> larger key; -0 is
-// taken as +0); 0 is reserved for "no entry".
-SP_DEVINL uint32_t fkey(float v) {
-  const uint32_t u = __float_as_uint(v + 0.0f);
-  return (u >> 31) ? ~u : (u | 0x80000000u);
-}
-SP_DEVINL float fkey_inv(uint32_t k) {
-  if (k == 0u) return -INFINITY;
-  return __uint_as_float((k >> 31) ? (k & 0x7FFFFFFFu) : ~k);
-}
-
-// Warp-wide selection of the best `per` of `tot` contiguous (value, index)
-// entries (value desc, index asc), E entries per lane at most; every lane gets
-// the result, best first.  Each pick is two redux.sync reductions: the largest
-// key, then the smallest index holding it.
-template <int GL, int E>
-SP_DEVINL void warp_merge_lists(const float* vin, const int* iin, int tot, int per, float (&out_v)[GL],
-                                int (&out_i)[GL]) {
-  const int lane = threadIdx.x & 31;
-  uint32_t key[E];
-  int ei[E];
-#pragma unroll
-  for (int k = 0; k < E; ++k) {
-    const int idx = lane + 32 * k;
-    key[k] = 0u;
-    ei[k] = INT_MAX;
-    if (idx < tot) {
-      ei[k] = iin[idx];
-      if (ei[k] != INT_MAX) key[k] = fkey(vin[idx]);
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < GL; ++r) {
-    out_v[r] = -INFINITY;
-    out_i[r] = INT_MAX;
-    if (r < per) {
-      uint32_t bk = key[0];
-      int bi = ei[0];
-#pragma unroll
-      for (int k = 1; k < E; ++k)
-        if (key[k] > bk || (key[k] == bk && ei[k] < bi)) { bk = key[k]; bi = ei[k]; }
-      const uint32_t mk = __reduce_max_sync(0xffffffffu, bk);
-      const int mi = (int)__reduce_min_sync(0xffffffffu, bk == mk ? (uint32_t)bi : 0x7fffffffu);
-      out_v[r] = fkey_inv(mk);
-      out_i[r] = mk ? mi : INT_MAX;
-#pragma unroll
-      for (int k = 0; k < E; ++k)
-        if (ei[k] == mi) { key[k] = 0u; ei[k] = INT_MAX; }
-    }
   }
 }
 

@@ -5,6 +5,7 @@ import pytest
 from oracle import core as O
 from paper_2609_13804_gb300 import synth as S
 import _parity as PT
+import test_gpu_parity as GP
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -45,4 +46,39 @@ def test_encoder_row_forms(B, D):
         ref = O.encoder(inp["X"][v0:v0 + n], Et, sel, s.enc_heads, s.ln_eps, store="bf16")
         assert np.abs(got[v0:v0 + n] - ref).max() <= PT.HID_MAX_ABS * np.sqrt((ref ** 2).mean())
         v0, t0 = v0 + n, t0 + t
+    selector.close()
+
+
+@pytest.mark.parametrize("n_vis,h,g,k_max,group", [
+    ([1, 126, 2, 127], 128, 1, 8, 0),          # one row tile, its last row and one more
+    ([254, 255, 31], 256, 1, 40, 0),           # the edges of one column tile
+    ([509, 33], 512, 1, 96, 0),                # history registers at their smaller capacity
+    ([330], 1024, 1, 223, 0),                  # and at the larger one
+    ([1016, 700], 128, 5, 120, 0),             # the widest slices, grouped rounds
+    ([64, 300], 128, 16, 100, 100),            # candidate groups, the longest lists
+])
+def test_selection_tables(B, n_vis, h, g, k_max, group):
+    """The table-driven selection at the edges of its tiles, slices and lists, with LN2's gain and bias."""
+    w = S.tiny_workload(93, n_vis, [1] * len(n_vis), D=128, D_text=128, h=h, enc_head_dim=64, k_max=k_max,
+                        group_size=group, g=g)
+    GP._run_select_case(B, w, scale=4.0 if h <= 256 else 2.0)
+
+
+def test_selection_tables_and_keys_agree(B):
+    """A workspace without room for the tables takes the general kernel: the same selection."""
+    w = S.tiny_workload(95, [700, 650], [1, 1], D=128, D_text=128, h=128, k_max=48)
+    s = S.SelectorShape(D=128, D_text=128, h=128, n_enc_layers=0)
+    selector = B.Selector(s, PT.scale_decoder(S.make_selector_weights(w, ln_affine=True), 4.0), DEV)
+    H, bias = B.dev_f32(S.make_memory(w), DEV), B.dev_f32(np.full(2, -1e30, np.float32), DEV)
+    full = B.sp_select(selector, w.n_vis, w.n_txt, H=H, stop_bias=bias, k_max=48)
+    rows = sum(w.n_vis) + 2  # what the general kernel carves, 256-byte slices
+    need = 4 * rows * (128 + 128 + 2 * 128 + 3 * 128) + 2 * rows * 3 * 128 + 4 * 2 * 1024 + 16 * 256
+    assert need < full["_ws"].numel()
+    small = B.sp_select(selector, w.n_vis, w.n_txt, H=H, stop_bias=bias, k_max=48, ws=full["_ws"][:need].clone())
+    torch.cuda.synchronize()
+    assert int(full["err"].item()) == 0 and int(small["err"].item()) == 0
+    assert (full["margin"][:, :48] > 1e-4).all()
+    np.testing.assert_array_equal(np_(full["order"]), np_(small["order"]))
+    g0, g1 = np_(full["gap"])[:, :48], np_(small["gap"])[:, :48]
+    assert np.abs(g0 - g1).max() <= 2e-4 * max(1.0, np.abs(g1).max())
     selector.close()
