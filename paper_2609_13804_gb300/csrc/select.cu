@@ -336,10 +336,21 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
     }
     __syncthreads();
   };
+  // The block's n results (staged in wpart_o, n a multiple of 4) into dst of
+  // every CTA, 16 bytes a lane: as 4-byte stores of the lanes that hold them,
+  // one peer each, the exchange was bound by its packets.
+  auto push_rows = [&](float* dst, int n) {
+    __syncthreads();
+    const int n4 = n >> 2;
+    for (int i = tid; i < n4 * C; i += NT) {
+      const int r = i / n4, c = i - r * n4;
+      *reinterpret_cast<float4*>(cluster.map_shared_rank(dst, r) + 4 * c) = reinterpret_cast<const float4*>(wpart_o)[c];
+    }
+  };
   // rows [rank R / C, +R / C) of W [R, h] (fp32) times the shared vector x;
   // half a warp per row, MR rows per half-warp at a time (their loads in
-  // flight together; each row's sum in the same order whatever MR is); each
-  // result is pushed into dst[row] of every CTA
+  // flight together; each row's sum in the same order whatever MR is); the
+  // results are pushed into dst of every CTA
   constexpr int MR = 4;
   auto matvec_f32_push = [&](const float* W, int R, const float* x, float* dst) {
     const int Rc = R / C, r0 = rank * Rc, hl = lane & 15, hw = lane >> 4;
@@ -366,12 +377,13 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
 #pragma unroll
         for (int i = 0; i < MR; ++i) sv[i] += __shfl_xor_sync(0xffffffffu, sv[i], o);
       }
-      if (hl < C) {
+      if (hl == 0) {
 #pragma unroll
         for (int i = 0; i < MR; ++i)
-          if (rb + i < Rc) *cluster.map_shared_rank(dst + r0 + rb + i, hl) = sv[i];
+          if (rb + i < Rc) wpart_o[rb + i] = sv[i];
       }
     }
+    push_rows(dst + r0, Rc);
   };
   // the same for W [R, K] in bf16, optionally through the exact GELU
   auto matvec_bf16_push = [&](const __nv_bfloat16* W, int R, int K, const float* x, float* dst, bool act) {
@@ -411,14 +423,29 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
 #pragma unroll
         for (int i = 0; i < MR; ++i) sv[i] = gelu_erf(sv[i]);
       }
-      if (hl < C) {
+      if (hl == 0) {
 #pragma unroll
         for (int i = 0; i < MR; ++i)
-          if (rb + i < Rc) *cluster.map_shared_rank(dst + r0 + rb + i, hl) = sv[i];
+          if (rb + i < Rc) wpart_o[rb + i] = sv[i];
       }
     }
+    push_rows(dst + r0, Rc);
   };
 
+  // this thread's DPT consecutive elements of an h-vector into v of every CTA,
+  // one vector store per peer
+  auto push_vec = [&](float* v, const float (&acc)[DPT]) {
+    for (int r = 0; r < C; ++r) {
+      float* dst = cluster.map_shared_rank(v, r) + el(0);
+      if (DPT == 4)
+        *reinterpret_cast<float4*>(dst) = make_float4(acc[0], acc[DPT > 1 ? 1 : 0], acc[DPT > 2 ? 2 : 0],
+                                                      acc[DPT > 3 ? 3 : 0]);
+      else if (DPT == 2)
+        *reinterpret_cast<float2*>(dst) = make_float2(acc[0], acc[DPT > 1 ? 1 : 0]);
+      else
+        dst[0] = acc[0];
+    }
+  };
   // this CTA's attention partial (max, sum, weighted values) from its warps'
   // partials, pushed into slot `slot` of every CTA (as in step 1 below)
   auto push_partial = [&](float4 (&o_w)[HV], float m_w, float l_w, int slot) {
@@ -438,14 +465,15 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
 #pragma unroll
     for (int w = 0; w < NW; ++w) cw[w] = __shfl_sync(0xffffffffu, cwl, w);
     float* sl = all_o + ((size_t)slot * C + rank) * h;
+    if (el(0) < h) {
+      float acc[DPT];
 #pragma unroll
-    for (int d = 0; d < DPT; ++d) {
-      const int i = el(d);
-      if (i >= h) continue;
-      float acc = 0.f;
+      for (int d = 0; d < DPT; ++d) {
+        acc[d] = 0.f;
 #pragma unroll
-      for (int w = 0; w < NW; ++w) acc += cw[w] * wpart_o[w * h + i];
-      for (int r = 0; r < C; ++r) *cluster.map_shared_rank(sl + i, r) = acc;
+        for (int w = 0; w < NW; ++w) acc[d] += cw[w] * wpart_o[w * h + el(d)];
+      }
+      push_vec(sl, acc);
     }
     if (tid < C) {
       float* ml = cluster.map_shared_rank(all_ml + ((size_t)slot * C + rank) * 2, tid);
@@ -798,17 +826,7 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
 #pragma unroll
           for (int w = 0; w < NW; ++w) acc[d] += cw[w] * wpart_o[w * h + el(d)];
         }
-        // one vector store per peer (DPT consecutive elements)
-        for (int r = 0; r < C; ++r) {
-          float* dst = cluster.map_shared_rank(slot, r) + el(0);
-          if (DPT == 4)
-            *reinterpret_cast<float4*>(dst) = make_float4(acc[0], acc[DPT > 1 ? 1 : 0], acc[DPT > 2 ? 2 : 0],
-                                                          acc[DPT > 3 ? 3 : 0]);
-          else if (DPT == 2)
-            *reinterpret_cast<float2*>(dst) = make_float2(acc[0], acc[DPT > 1 ? 1 : 0]);
-          else
-            dst[0] = acc[0];
-        }
+        push_vec(slot, acc);
       }
       if (tid < C) {
         float* ml = cluster.map_shared_rank(all_ml + ((size_t)buf * C + rank) * 2, tid);
@@ -1166,6 +1184,13 @@ restore_kernel(const BatchDesc bd, const int* order, const int* ep_count,
 
 }  // namespace
 
+// Episodes that all run at once as 16-CTA clusters (one per GPC).  A round of a
+// decoder of several layers streams the lower layers' weights and cross-attention
+// rows from L2 through its cluster's SMs: with half the rows per CTA 4 episodes
+// of 576 take 50 us a round in place of 62 (16-byte pushes of the mat-vecs' and
+// partials' results included).
+constexpr int kWideClusters = 8;
+
 int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_smem, size_t* smem_bytes, bool multi) {
   int n_max = 0;
   for (int b = 0; b < bd.B; ++b) {
@@ -1173,7 +1198,9 @@ int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_sme
     n_max = std::max(n_max, bd.group_size > 0 ? std::min(bd.group_size, n) : n);
   }
   const size_t budget = 225 * 1024;
+  const int n_ep = bd.ep_off[bd.B];
   for (int C : {8, 16}) {
+    if (C == 8 && multi && n_ep <= kWideClusters) continue;
     const int n_loc = (n_max + C - 1) / C;
     const size_t need = sel_layout(h, n_loc, k_max, C, true, multi).total;
     if (n_loc + 1 <= 128 && need <= budget) {  // the dims-major logits take <= 128 columns
