@@ -60,7 +60,7 @@ __host__ __device__ inline SelSmem sel_layout(int h, int n_loc, int k_max, int C
   // keys in shared memory: dims-major, (n_loc + 1) columns (the last one is
   // STOP's key), float4 (d4, j) at d4 * (n_loc + 1) + j
   L.kt = o;       o += al16(keys_in_smem ? (size_t)(n_loc + 1) * h * 4 : 0);
-  L.lgp = o;      o += al16(keys_in_smem ? (size_t)NW * (n_loc + 1) * 4 : 0);
+  L.lgp = o;      o += al16((size_t)(keys_in_smem ? NW * (n_loc + 1) : n_loc) * 4);
   L.stopkt = o;   o += al16((size_t)h * 4);
   L.wpart_o = o;  o += al16((size_t)NW * h * 4);
   L.wpart_ml = o; o += al16((size_t)NW * 2 * 4);
@@ -130,40 +130,6 @@ SP_DEVINL void block_sum_n(float (&v)[U], float* red) {
 
 SP_DEVINL float dot4(const float4& a, const float4& b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 
-// Keeps the best `keep` (value, index) pairs seen so far, best first, in a list
-// of capacity GL.  All lanes of a warp hold the same list.
-template <int GL>
-SP_DEVINL void top_insert(float (&tv)[GL], int (&ti)[GL], float v, int j, int keep) {
-  // the current last kept entry, selected with compile-time indices only so the
-  // list stays in registers
-  float lv = tv[0];
-  int li = ti[0];
-#pragma unroll
-  for (int k = 1; k < GL; ++k) {
-    if (k == keep - 1) {
-      lv = tv[k];
-      li = ti[k];
-    }
-  }
-  if (!better(v, j, lv, li)) return;
-#pragma unroll
-  for (int k = GL - 1; k > 0; --k) {
-    if (k < keep) {
-      if (better(v, j, tv[k - 1], ti[k - 1])) {
-        tv[k] = tv[k - 1];
-        ti[k] = ti[k - 1];
-      } else if (better(v, j, tv[k], ti[k])) {
-        tv[k] = v;
-        ti[k] = j;
-      }
-    }
-  }
-  if (better(v, j, tv[0], ti[0])) {
-    tv[0] = v;
-    ti[0] = j;
-  }
-}
-
 // HV = h / 128: float4 slices per lane of an h-vector (lane holds elements
 // 4 (lane + 32 k) .. +3, k < HV).  GL = capacity of the per-round top lists
 // (g + 1 <= GL).  P = history positions a warp loads at once.
@@ -177,7 +143,7 @@ __global__ void __launch_bounds__(NT, 1)
 select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in_smem, int tm_cols) {
   constexpr int P = (16 / HV) > 0 ? 16 / HV : 1;
   constexpr int DPT = (HV * 128) / NT > 0 ? (HV * 128) / NT : 1;  // dims per thread in the merges
-  constexpr int U = 4;                                          // candidates per warp iteration
+  constexpr int U = 4;  // candidates per warp iteration
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks();
   const int rank = (int)cluster.block_rank();
@@ -953,21 +919,55 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
       }
     } else {
       for (int jb = warp * U; jb < nl; jb += NW * U) {
-        float sv[U];
-        bool ok[U];
+        float4 kr[U][HV];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int j = jb + u;
-          ok[u] = j < nl && !taken[j];
-          sv[u] = 0.f;
-          const float4* kr = reinterpret_cast<const float4*>(KT + (size_t)(row0 + j0 + min(j, nl - 1)) * a.ldkt);
+          const float4* kp = reinterpret_cast<const float4*>(KT + (size_t)(row0 + j0 + min(jb + u, nl - 1)) * a.ldkt);
 #pragma unroll
-          for (int k = 0; k < HV; ++k) sv[u] += dot4(xr[k], __ldg(kr + lane + 32 * k));
+          for (int k = 0; k < HV; ++k) kr[u][k] = __ldg(kp + lane + 32 * k);
+        }
+        float sv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          sv[u] = 0.f;
+#pragma unroll
+          for (int k = 0; k < HV; ++k) sv[u] += dot4(xr[k], kr[u][k]);
         }
         warp_sum_n<U>(sv);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          if (ok[u]) top_insert<GL>(tv, ti, sv[u], j0 + jb + u, per);
+          if (lane == u && jb + u < nl) lgp[jb + u] = sv[u];
+      }
+      __syncthreads();
+      // this warp's top g+1: lane's candidates tid + 256 i.  (One list per warp
+      // kept by insertion in all its lanes took 150 instructions a row: 20 us a
+      // round of 4 x 3,328 candidates with g = 5, 16 now; keeping a third of the
+      // rows in shared memory gives nothing more.)
+      uint32_t key[SP_MAX_NVIS / 16 / NT];
+      int id[SP_MAX_NVIS / 16 / NT];
+#pragma unroll
+      for (int i = 0; i < SP_MAX_NVIS / 16 / NT; ++i) {
+        const int j = tid + NT * i;
+        const bool ok = j < nl && !taken[j];
+        key[i] = ok ? fkey(lgp[j]) : 0u;
+        id[i] = ok ? j0 + j : INT_MAX;
+      }
+#pragma unroll
+      for (int r = 0; r < GL; ++r) {
+        if (r < per) {
+          uint32_t bk = key[0];
+          int bi = id[0];
+#pragma unroll
+          for (int i = 1; i < SP_MAX_NVIS / 16 / NT; ++i)
+            if (key[i] > bk) { bk = key[i]; bi = id[i]; }  // (indices ascend with i)
+          const uint32_t mk = __reduce_max_sync(0xffffffffu, bk);
+          const int mi = (int)__reduce_min_sync(0xffffffffu, bk == mk ? (uint32_t)bi : 0x7fffffffu);
+          tv[r] = fkey_inv(mk);
+          ti[r] = mk ? mi : INT_MAX;
+#pragma unroll
+          for (int i = 0; i < SP_MAX_NVIS / 16 / NT; ++i)
+            if (id[i] == mi) { key[i] = 0u; id[i] = INT_MAX; }
+        }
       }
       float s1[1] = {0.f};
 #pragma unroll
@@ -1064,19 +1064,21 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
       if (a.gap) a.gap[trace + round] = best - stop_raw;
       if (a.margin) {
         // smallest gap between consecutive values among the top g+1 of
-        // {available visual logits} U {STOP}
-        float vals[GMAX + 2];
-        int n = 0;
+        // {available visual logits} U {STOP}: STOP bubbles down the list
         const int nv = min(per, n_avail);
-        for (int k = 0; k < nv; ++k) vals[n++] = gtop_v[k];
-        int ins = n;
-        while (ins > 0 && vals[ins - 1] < stop_logit) --ins;
-        for (int k = n; k > ins; --k) vals[k] = vals[k - 1];
-        vals[ins] = stop_logit;
-        ++n;
-        const int use = min(n, per);
-        float mg = INFINITY;
-        for (int k = 0; k + 1 < use; ++k) mg = fminf(mg, vals[k] - vals[k + 1]);
+        const int use = min(nv + 1, per);
+        float mg = INFINITY, c = stop_logit, prev = 0.f;
+#pragma unroll
+        for (int k = 0; k <= GL; ++k) {
+          float x = c;
+          if (k < GL && k < nv) {
+            const float tk = gtop_v[k];
+            x = fmaxf(tk, c);
+            c = fminf(tk, c);
+          }
+          if (k > 0 && k < use) mg = fminf(mg, prev - x);
+          prev = x;
+        }
         a.margin[trace + round] = mg;
       }
     }
@@ -1190,6 +1192,7 @@ restore_kernel(const BatchDesc bd, const int* order, const int* ep_count,
 // of 576 take 50 us a round in place of 62 (16-byte pushes of the mat-vecs' and
 // partials' results included).
 constexpr int kWideClusters = 8;
+constexpr size_t kSmemBudget = 225 * 1024;
 
 int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_smem, size_t* smem_bytes, bool multi) {
   int n_max = 0;
@@ -1197,13 +1200,12 @@ int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_sme
     const int n = bd.vis_off[b + 1] - bd.vis_off[b];
     n_max = std::max(n_max, bd.group_size > 0 ? std::min(bd.group_size, n) : n);
   }
-  const size_t budget = 225 * 1024;
   const int n_ep = bd.ep_off[bd.B];
   for (int C : {8, 16}) {
     if (C == 8 && multi && n_ep <= kWideClusters) continue;
     const int n_loc = (n_max + C - 1) / C;
     const size_t need = sel_layout(h, n_loc, k_max, C, true, multi).total;
-    if (n_loc + 1 <= 128 && need <= budget) {  // the dims-major logits take <= 128 columns
+    if (n_loc + 1 <= 128 && need <= kSmemBudget) {  // the dims-major logits take <= 128 columns
       *keys_in_smem = true;
       *smem_bytes = need;
       return C;

@@ -6,8 +6,6 @@
 
 namespace sp {
 
-SP_DEVINL bool better(float v, int i, float bv, int bi) { return v > bv || (v == bv && i < bi); }
-
 // Order-preserving 32-bit key of a float (larger float -> larger key; -0 is
 // taken as +0); 0 is reserved for "no entry".
 SP_DEVINL uint32_t fkey(float v) {
