@@ -461,7 +461,7 @@ size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* ou
 
 // Whether the selection goes through per-episode tables.  They cost kGramFixedUs
 // and 30 h (n + 2)^2 tensor operations per episode (16 x 576 candidates, h = 512:
-// 155 us with their operands, 0.53e9 a microsecond; one of 576, h = 256: 23 us)
+// 140 us with their operands, 0.59e9 a microsecond; one of 576, h = 256: 23 us)
 // and save kGramRoundUs of every round (16 x 576: 4.9 -> 2.5 us; training 6.8 ->
 // 2.6; one image 5.6 -> 2.1); the rounds are bounded by the cap (a STOP can end
 // them early, which only the device knows).

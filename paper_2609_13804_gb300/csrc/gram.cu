@@ -154,13 +154,16 @@ gram_operands_kernel(const BatchDesc bd, const GramArgs g) {
 }
 
 // ---- tables
-// Persistent kernel, one CTA per SM, 6 warps as in the GEMM: TMA producer, MMA
-// issuer, four epilogue warps; two fp32 accumulators (large and small products)
+// Persistent kernel, one CTA per SM, 10 warps: TMA producer, MMA issuer, eight
+// epilogue warps (two per TMEM lane quadrant, every other 32 columns); two fp32 accumulators (large and small products)
 // fill TMEM, so a tile's epilogue runs between its MMAs and the next tile's.  A
 // work item is one 128 x n_tile tile of one table of one episode.  A stage
 // holds both parts of 64 columns of both operands and feeds all three products
 // (12 MMAs of K = 16): 85 KB for 1,250 tensor cycles at n_tile 208, 68 B/cycle,
 // where staging the products one by one as a GEMM over 3h would take 101.
+// 16 episodes of 576, h = 512 (82 useful GFLOP of three products, 107 MB of
+// tables): 112 us (126 with four epilogue warps), bound by the loads' latency at
+// two stages and by the epilogue that nothing overlaps.
 constexpr int BM = 128;
 constexpr int BK = 64;
 constexpr int STAGES = 2;
@@ -168,7 +171,9 @@ constexpr int NMAX = 256;
 constexpr uint32_t A_BYTES = BM * BK * 2;
 constexpr uint32_t B_BYTES = NMAX * BK * 2;
 constexpr uint32_t STAGE_BYTES = 2 * (A_BYTES + B_BYTES);
-constexpr uint32_t EPI_BYTES = 4 * 32 * 33 * 4;
+constexpr int EPI_WARPS = 8;
+constexpr int GT = 64 + 32 * EPI_WARPS;
+constexpr uint32_t EPI_BYTES = EPI_WARPS * 32 * 33 * 4;
 constexpr size_t GRAM_SMEM = 1024 + STAGES * STAGE_BYTES + EPI_BYTES + 256;
 
 struct Tile {
@@ -194,7 +199,7 @@ SP_DEVINL bool tile_of(const BatchDesc& bd, const GramArgs& g, int t, Tile& o) {
 SP_DEVINL int a_mat(int p) { return (0x32432 >> (4 * p)) & 15; }  // vc zc QS vc zc
 SP_DEVINL int b_mat(int p) { return (0x22100 >> (4 * p)) & 15; }  // KTg KTg KS vc vc
 
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(GT, 1)
 gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const BatchDesc bd,
             const GramArgs g) {
   extern __shared__ uint8_t smem_raw[];
@@ -215,7 +220,7 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       mbar_init(&empty[s], 1);
     }
     mbar_init(tfull, 1);
-    mbar_init(tempty, 4);
+    mbar_init(tempty, EPI_WARPS);
     mbar_init(done, 1);
     fence_mbar_init();
     tma_prefetch_desc(&tmA);
@@ -293,7 +298,7 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     __syncwarp();
   } else {
     const int quad = warp & 3;
-    float* st = stg + quad * 32 * 33;
+    float* st = stg + (warp - 2) * 32 * 33;
     int it = 0;
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
       Tile w;
@@ -311,7 +316,7 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
       const int rows = min(32, np - i0);
       if (rows > 0) {
-        for (int c = 0; c < cols; c += 32) {
+        for (int c = ((warp - 2) >> 2) * 32; c < cols; c += EPI_WARPS * 8) {
           float v[32], u[32];
           tmem_ld_32x32b_x32(taddr + c, v);
           tmem_ld_32x32b_x32(taddr + NMAX + c, u);
@@ -321,9 +326,17 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           __syncwarp();
           const bool live = c + lane < cols;
           const float ib = live ? inv_b[c + lane] : 0.f;
-#pragma unroll 8
-          for (int r = 0; r < 32; ++r)
-            if (live && r < rows) out[(size_t)r * (5 * g.ld) + c + lane] = st[r * 33 + lane] * ib;
+          float* o = out + c + lane;
+          if (rows == 32) {
+#pragma unroll 16
+            for (int r = 0; r < 32; ++r, o += 5 * g.ld) {
+              const float x = st[r * 33 + lane] * ib;
+              if (live) *o = x;
+            }
+          } else {
+            for (int r = 0; r < rows; ++r, o += 5 * g.ld)
+              if (live) *o = st[r * 33 + lane] * ib;
+          }
           __syncwarp();
         }
       }
@@ -386,7 +399,7 @@ cudaError_t gram_launch(const BatchDesc& bd, const GramArgs& g, cudaStream_t st)
     }
   }
   prof_begin_launch(st);
-  r = launch_pdl(gram_kernel, dim3(std::min(tiles, device_sm_count())), dim3(192), GRAM_SMEM, st, ta, tb, bd, g);
+  r = launch_pdl(gram_kernel, dim3(std::min(tiles, device_sm_count())), dim3(GT), GRAM_SMEM, st, ta, tb, bd, g);
   prof_end_launch(st, SP_K_SGEMM, flops, 0.0);
   return r;
 }
