@@ -130,6 +130,164 @@ SP_DEVINL void block_sum_n(float (&v)[U], float* red) {
 
 SP_DEVINL float dot4(const float4& a, const float4& b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 
+// ---- decoders of several layers: the mat-vecs and the cross-attention are
+// functions of their own, so that each has the whole register file for the rows
+// it keeps in flight (inlined, their loads were serialised by the register
+// pressure of the selection round: a batch of loads took 2,500 to 3,000 cycles).
+
+// res[0, Rc) = rows [r0, r0 + Rc) of W [., h] (fp32) times the shared vector x;
+// half a warp per row, MR rows per half-warp in flight (each row's sum in the
+// same order whatever MR is).
+template <int MR>
+__device__ __noinline__ void matvec_f32(const float* W, int r0, int Rc, int h, const float* x, float* res) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hl = lane & 15, hw = lane >> 4;
+  const int cu = h / 4;  // float4 chunks per row
+  const float4* x4 = reinterpret_cast<const float4*>(x);
+  for (int rb = (warp * 2 + hw) * MR; rb < Rc; rb += NW * 2 * MR) {
+    const float4* wr[MR];
+    float sv[MR];
+#pragma unroll
+    for (int i = 0; i < MR; ++i) {
+      wr[i] = reinterpret_cast<const float4*>(W + (size_t)(r0 + min(rb + i, Rc - 1)) * h);
+      sv[i] = 0.f;
+    }
+#pragma unroll 4
+    for (int u = hl; u < cu; u += 16) {
+      const float4 xv = x4[u];
+      float4 wv[MR];
+#pragma unroll
+      for (int i = 0; i < MR; ++i) wv[i] = __ldg(wr[i] + u);
+#pragma unroll
+      for (int i = 0; i < MR; ++i) sv[i] += dot4(xv, wv[i]);
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+#pragma unroll
+      for (int i = 0; i < MR; ++i) sv[i] += __shfl_xor_sync(hw ? 0xffff0000u : 0x0000ffffu, sv[i], o);
+    }
+    if (hl == 0) {
+#pragma unroll
+      for (int i = 0; i < MR; ++i)
+        if (rb + i < Rc) res[rb + i] = sv[i];
+    }
+  }
+}
+
+// The same for W [., K] in bf16, optionally through the exact GELU.
+template <int MR>
+__device__ __noinline__ void matvec_bf16(const __nv_bfloat16* W, int r0, int Rc, int K, const float* x, float* res,
+                                         bool act) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hl = lane & 15, hw = lane >> 4;
+  const int cu = K / 8;  // 8-element chunks per row
+  const float4* x4 = reinterpret_cast<const float4*>(x);
+  for (int rb = (warp * 2 + hw) * MR; rb < Rc; rb += NW * 2 * MR) {
+    const uint4* wr[MR];
+    float sv[MR];
+#pragma unroll
+    for (int i = 0; i < MR; ++i) {
+      wr[i] = reinterpret_cast<const uint4*>(W + (size_t)(r0 + min(rb + i, Rc - 1)) * K);
+      sv[i] = 0.f;
+    }
+#pragma unroll(MR >= 8 ? 4 : 16 / MR)
+    for (int u = hl; u < cu; u += 16) {
+      const float4 xa = x4[2 * u], xb = x4[2 * u + 1];
+      const float xs[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+      uint4 pw[MR];
+#pragma unroll
+      for (int i = 0; i < MR; ++i) pw[i] = __ldg(wr[i] + u);
+#pragma unroll
+      for (int i = 0; i < MR; ++i) {
+        const uint32_t q[4] = {pw[i].x, pw[i].y, pw[i].z, pw[i].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 f = unpack_bf16x2(q[k]);
+          sv[i] += f.x * xs[2 * k] + f.y * xs[2 * k + 1];
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+#pragma unroll
+      for (int i = 0; i < MR; ++i) sv[i] += __shfl_xor_sync(hw ? 0xffff0000u : 0x0000ffffu, sv[i], o);
+    }
+    float v = sv[0];  // lane i of the half-warp finishes row i
+#pragma unroll
+    for (int i = 1; i < MR; ++i)
+      if (hl == i) v = sv[i];
+    if (hl < MR && rb + hl < Rc) res[rb + hl] = act ? gelu_erf(v) : v;
+  }
+}
+
+// This warp's share of the cross-attention of the shared vector x over n rows
+// (row i: first + i, the last one `stop` if has_stop) of folded keys (h floats)
+// and values (the next h), PC rows in flight: its partial
+// (weighted values, max, sum) into o [h], ml [2].
+template <int HV>
+__device__ __noinline__ void cross_warp(const float* KC, int ld, int first, int n, int has_stop, int stop,
+                                        const float* x, float* o, float* ml) {
+  constexpr int PC = HV <= 4 ? 5 : 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float4 xv[HV], acc[HV];
+#pragma unroll
+  for (int k = 0; k < HV; ++k) {
+    xv[k] = reinterpret_cast<const float4*>(x)[lane + 32 * k];
+    acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  float m = -INFINITY, l = 0.f;
+  for (int k0 = warp * PC; k0 < n; k0 += NW * PC) {
+    const float4* row[PC];
+    float4 r[PC][HV];
+#pragma unroll
+    for (int p = 0; p < PC; ++p) {
+      const int i = min(k0 + p, n - 1);
+      row[p] = reinterpret_cast<const float4*>(KC + (size_t)(has_stop && i == n - 1 ? stop : first + i) * ld) + lane;
+#pragma unroll
+      for (int k = 0; k < HV; ++k) r[p][k] = __ldg(row[p] + 32 * k);
+    }
+    float sc[PC];
+#pragma unroll
+    for (int p = 0; p < PC; ++p) {
+      sc[p] = 0.f;
+#pragma unroll
+      for (int k = 0; k < HV; ++k) sc[p] += dot4(xv[k], r[p][k]);
+    }
+#pragma unroll
+    for (int p = 0; p < PC; ++p)  // the values, while the scores are reduced
+#pragma unroll
+      for (int k = 0; k < HV; ++k) r[p][k] = __ldg(row[p] + 32 * HV + 32 * k);
+    warp_sum_n<PC>(sc);
+    float mn = m;
+#pragma unroll
+    for (int p = 0; p < PC; ++p) {
+      if (k0 + p >= n) sc[p] = -INFINITY;
+      mn = fmaxf(mn, sc[p]);
+    }
+    const float cw = m == -INFINITY ? 0.f : __expf(m - mn);
+    l *= cw;
+#pragma unroll
+    for (int k = 0; k < HV; ++k) { acc[k].x *= cw; acc[k].y *= cw; acc[k].z *= cw; acc[k].w *= cw; }
+#pragma unroll
+    for (int p = 0; p < PC; ++p) {
+      const float ps = k0 + p < n ? __expf(sc[p] - mn) : 0.f;
+      l += ps;
+#pragma unroll
+      for (int k = 0; k < HV; ++k) {
+        acc[k].x = fmaf(ps, r[p][k].x, acc[k].x);
+        acc[k].y = fmaf(ps, r[p][k].y, acc[k].y);
+        acc[k].z = fmaf(ps, r[p][k].z, acc[k].z);
+        acc[k].w = fmaf(ps, r[p][k].w, acc[k].w);
+      }
+    }
+    m = mn;
+  }
+#pragma unroll
+  for (int k = 0; k < HV; ++k) reinterpret_cast<float4*>(o)[lane + 32 * k] = acc[k];
+  if (lane == 0) {
+    ml[0] = m;
+    ml[1] = l;
+  }
+}
+
 // HV = h / 128: float4 slices per lane of an h-vector (lane holds elements
 // 4 (lane + 32 k) .. +3, k < HV).  GL = capacity of the per-round top lists
 // (g + 1 <= GL).  P = history positions a warp loads at once.
@@ -313,88 +471,18 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
       *reinterpret_cast<float4*>(cluster.map_shared_rank(dst, r) + 4 * c) = reinterpret_cast<const float4*>(wpart_o)[c];
     }
   };
-  // rows [rank R / C, +R / C) of W [R, h] (fp32) times the shared vector x;
-  // half a warp per row, MR rows per half-warp at a time (their loads in
-  // flight together; each row's sum in the same order whatever MR is); the
-  // results are pushed into dst of every CTA
-  constexpr int MR = 4;
+  // this CTA's rows [rank R / C, +R / C) of a product, into dst of every CTA
   auto matvec_f32_push = [&](const float* W, int R, const float* x, float* dst) {
-    const int Rc = R / C, r0 = rank * Rc, hl = lane & 15, hw = lane >> 4;
-    const int cu = h / 4;  // float4 chunks per row
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    for (int rb = (warp * 2 + hw) * MR; rb < Rc; rb += NW * 2 * MR) {
-      const float4* wr[MR];
-#pragma unroll
-      for (int i = 0; i < MR; ++i) wr[i] = reinterpret_cast<const float4*>(W + (size_t)(r0 + min(rb + i, Rc - 1)) * h);
-      float sv[MR];
-#pragma unroll
-      for (int i = 0; i < MR; ++i) sv[i] = 0.f;
-#pragma unroll 4
-      for (int u = hl; u < cu; u += 16) {
-        const float4 xv = x4[u];
-        float4 wv[MR];
-#pragma unroll
-        for (int i = 0; i < MR; ++i) wv[i] = __ldg(wr[i] + u);
-#pragma unroll
-        for (int i = 0; i < MR; ++i) sv[i] += dot4(xv, wv[i]);
-      }
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {
-#pragma unroll
-        for (int i = 0; i < MR; ++i) sv[i] += __shfl_xor_sync(0xffffffffu, sv[i], o);
-      }
-      if (hl == 0) {
-#pragma unroll
-        for (int i = 0; i < MR; ++i)
-          if (rb + i < Rc) wpart_o[rb + i] = sv[i];
-      }
-    }
+    const int Rc = R / C, r0 = rank * Rc;
+    matvec_f32<6>(W, r0, Rc, h, x, wpart_o);
     push_rows(dst + r0, Rc);
   };
-  // the same for W [R, K] in bf16, optionally through the exact GELU
   auto matvec_bf16_push = [&](const __nv_bfloat16* W, int R, int K, const float* x, float* dst, bool act) {
-    const int Rc = R / C, r0 = rank * Rc, hl = lane & 15, hw = lane >> 4;
-    const int cu = K / 8;  // 8-element chunks per row
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    for (int rb = (warp * 2 + hw) * MR; rb < Rc; rb += NW * 2 * MR) {
-      const uint4* wr[MR];
-#pragma unroll
-      for (int i = 0; i < MR; ++i) wr[i] = reinterpret_cast<const uint4*>(W + (size_t)(r0 + min(rb + i, Rc - 1)) * K);
-      float sv[MR];
-#pragma unroll
-      for (int i = 0; i < MR; ++i) sv[i] = 0.f;
-#pragma unroll 4
-      for (int u = hl; u < cu; u += 16) {
-        const float4 xa = x4[2 * u], xb = x4[2 * u + 1];
-        const float xs[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-        uint4 pw[MR];
-#pragma unroll
-        for (int i = 0; i < MR; ++i) pw[i] = __ldg(wr[i] + u);
-#pragma unroll
-        for (int i = 0; i < MR; ++i) {
-          const uint32_t q[4] = {pw[i].x, pw[i].y, pw[i].z, pw[i].w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float2 f = unpack_bf16x2(q[k]);
-            sv[i] += f.x * xs[2 * k] + f.y * xs[2 * k + 1];
-          }
-        }
-      }
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {
-#pragma unroll
-        for (int i = 0; i < MR; ++i) sv[i] += __shfl_xor_sync(0xffffffffu, sv[i], o);
-      }
-      if (act) {
-#pragma unroll
-        for (int i = 0; i < MR; ++i) sv[i] = gelu_erf(sv[i]);
-      }
-      if (hl == 0) {
-#pragma unroll
-        for (int i = 0; i < MR; ++i)
-          if (rb + i < Rc) wpart_o[rb + i] = sv[i];
-      }
-    }
+    const int Rc = R / C, r0 = rank * Rc;
+    if (Rc > NW * 2 * 4)
+      matvec_bf16<8>(W, r0, Rc, K, x, wpart_o, act);
+    else  // (few rows: two per half-warp, more of each in flight)
+      matvec_bf16<2>(W, r0, Rc, K, x, wpart_o, act);
     push_rows(dst + r0, Rc);
   };
 
@@ -414,13 +502,7 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
   };
   // this CTA's attention partial (max, sum, weighted values) from its warps'
   // partials, pushed into slot `slot` of every CTA (as in step 1 below)
-  auto push_partial = [&](float4 (&o_w)[HV], float m_w, float l_w, int slot) {
-#pragma unroll
-    for (int k = 0; k < HV; ++k) reinterpret_cast<float4*>(wpart_o + warp * h)[lane + 32 * k] = o_w[k];
-    if (lane == 0) {
-      wpart_ml[warp * 2 + 0] = m_w;
-      wpart_ml[warp * 2 + 1] = l_w;
-    }
+  auto push_partial = [&](int slot) {  // (from wpart_o, wpart_ml)
     __syncthreads();
     const float mwl = lane < NW ? wpart_ml[lane * 2] : -INFINITY;
     const float lwl = lane < NW ? wpart_ml[lane * 2 + 1] : 0.f;
@@ -458,15 +540,28 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
 #pragma unroll
     for (int r = 0; r < 16; ++r) wr[r] = __shfl_sync(0xffffffffu, wrl, r);
 #pragma unroll
-    for (int d = 0; d < DPT; ++d) {
-      const int i = el(d);
-      out[d] = 0.f;
-      if (i >= h) continue;
-      float o = 0.f;
+    for (int d = 0; d < DPT; ++d) out[d] = 0.f;
+    if (el(0) < h) {
+      const float* sl = all_o + (size_t)slot * C * h + el(0);
 #pragma unroll
-      for (int r = 0; r < 16; ++r)
-        if (r < C) o += wr[r] * all_o[((size_t)slot * C + r) * h + i];
-      out[d] = o * inv;
+      for (int r = 0; r < 16; ++r) {
+        if (r < C) {
+          float v[DPT];
+          if (DPT == 4) {
+            const float4 x = *reinterpret_cast<const float4*>(sl + r * h);
+            v[0] = x.x; v[DPT > 1 ? 1 : 0] = x.y; v[DPT > 2 ? 2 : 0] = x.z; v[DPT > 3 ? 3 : 0] = x.w;
+          } else if (DPT == 2) {
+            const float2 x = *reinterpret_cast<const float2*>(sl + r * h);
+            v[0] = x.x; v[DPT > 1 ? 1 : 0] = x.y;
+          } else {
+            v[0] = sl[r * h];
+          }
+#pragma unroll
+          for (int d = 0; d < DPT; ++d) out[d] += wr[r] * v[d];
+        }
+      }
+#pragma unroll
+      for (int d = 0; d < DPT; ++d) out[d] *= inv;
     }
   };
   constexpr int PL = P > 1 ? P / 2 : 1;  // rows per warp batch in the deep-decoder loops
@@ -539,49 +634,21 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
       warp_sum_n<PL>(sc);
       absorb(sc, vr, np2 - k0, m_w, l_w, o_w);
     }
-    push_partial(o_w, m_w, l_w, slot);
+#pragma unroll
+    for (int k = 0; k < HV; ++k) reinterpret_cast<float4*>(wpart_o + warp * h)[lane + 32 * k] = o_w[k];
+    if (lane == 0) {
+      wpart_ml[warp * 2 + 0] = m_w;
+      wpart_ml[warp * 2 + 1] = l_w;
+    }
+    push_partial(slot);
   };
   // layer l's cross-attention of the normalised input mn over every row of the
   // episode's memory (this CTA's candidate slice; rank 0 adds the STOP row),
   // with the folded keys (Wq_c^T Wk_c m / sqrt h) and values (Wo_c Wv_c m)
   auto cross_partial = [&](int l, int slot) {
-    float4 xv[HV];
-#pragma unroll
-    for (int k = 0; k < HV; ++k) xv[k] = reinterpret_cast<const float4*>(mn)[lane + 32 * k];
-    const float* KCl = a.KC + (size_t)2 * l * h;
-    const int ncand = nl + (rank == 0 ? 1 : 0);
-    float m_w = -INFINITY, l_w = 0.f;
-    float4 o_w[HV];
-#pragma unroll
-    for (int k = 0; k < HV; ++k) o_w[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k0 = warp * PL; k0 < ncand; k0 += NW * PL) {
-      float4 kr[PL][HV], vr[PL][HV];
-#pragma unroll
-      for (int pp = 0; pp < PL; ++pp) {
-        if (k0 + pp < ncand) {
-          const int jj = k0 + pp;
-          const int row = jj < nl ? row0 + j0 + jj : a.stop_row;
-          const float4* kc = reinterpret_cast<const float4*>(KCl + (size_t)row * a.ldz);
-#pragma unroll
-          for (int k = 0; k < HV; ++k) {
-            kr[pp][k] = __ldg(kc + lane + 32 * k);
-            vr[pp][k] = __ldg(kc + h / 4 + lane + 32 * k);
-          }
-        }
-      }
-      float sc[PL];
-#pragma unroll
-      for (int pp = 0; pp < PL; ++pp) {
-        sc[pp] = 0.f;
-        if (k0 + pp < ncand) {
-#pragma unroll
-          for (int k = 0; k < HV; ++k) sc[pp] += dot4(xv[k], kr[pp][k]);
-        }
-      }
-      warp_sum_n<PL>(sc);
-      absorb(sc, vr, ncand - k0, m_w, l_w, o_w);
-    }
-    push_partial(o_w, m_w, l_w, slot);
+    cross_warp<HV>(a.KC + (size_t)2 * l * h, a.ldz, row0 + j0, nl + (rank == 0 ? 1 : 0), rank == 0, a.stop_row, mn,
+                   wpart_o + warp * h, wpart_ml + warp * 2);
+    push_partial(slot);
   };
 
   float alive = 1.f, disc = a.beta, kbar_acc = 0.f;  // A_t, beta^t, Eq. 7 (TRAIN)
@@ -1189,8 +1256,8 @@ restore_kernel(const BatchDesc bd, const int* order, const int* ep_count,
 // Episodes that all run at once as 16-CTA clusters (one per GPC).  A round of a
 // decoder of several layers streams the lower layers' weights and cross-attention
 // rows from L2 through its cluster's SMs: with half the rows per CTA 4 episodes
-// of 576 take 50 us a round in place of 62 (16-byte pushes of the mat-vecs' and
-// partials' results included).
+// of 576 take 42 us a round in place of 62 (the pushes of 16 bytes a lane and the
+// row batches of the functions above included).
 constexpr int kWideClusters = 8;
 constexpr size_t kSmemBudget = 225 * 1024;
 
