@@ -1320,8 +1320,9 @@ struct PipeParts {
   size_t scratch_bytes;
 };
 
+// tables: with room for the selection's tables where its plan has them
 size_t pipe_ws(const sp_selector* s, const sp_model* m, const sp_select_in& sel, const PipePlan& pp, Carve& cv,
-               PipeParts* out) {
+               PipeParts* out, bool tables = true) {
   PipeParts q;
   q.packed = cv.take<uint16_t>((size_t)std::max(pp.T_cap, 1) * m->cfg.d);
   q.pos = cv.take<int>((size_t)std::max(pp.T_cap, 1));
@@ -1333,6 +1334,7 @@ size_t pipe_ws(const sp_selector* s, const sp_model* m, const sp_select_in& sel,
   sp_select_in si = sel;
   si.H = nullptr;
   plan_select(s, &si, &sp_);
+  if (!tables) sp_.gram_C = 0;
   Carve c1(nullptr), c2(nullptr), c3(nullptr);
   sp_select_out so = {};
   so.order = nullptr;
@@ -1368,7 +1370,11 @@ static sp_status pipeline_impl(const sp_selector* s, const sp_model* m, const sp
   if (!io->idx || !io->count || !io->cu_seqlens || !io->hidden) return fail(SP_ERR_INVALID_ARG, "sp_pipeline: idx, count, cu_seqlens, hidden required");
   Carve cv(ws);
   PipeParts q;
-  const size_t need = pipe_ws(s, m, io->sel, pp, cv, &q) + 256;
+  size_t need = pipe_ws(s, m, io->sel, pp, cv, &q) + 256;
+  if (ws && ws_bytes < need) {  // without room for the tables: the general selection kernel
+    cv = Carve(ws);
+    need = pipe_ws(s, m, io->sel, pp, cv, &q, false) + 256;
+  }
   if (!ws || ws_bytes < need) return fail(SP_ERR_WORKSPACE, "sp_pipeline: workspace %zu < %zu bytes", ws_bytes, need);
   if (!al16(ws)) return fail(SP_ERR_ALIGN, "sp_pipeline: workspace must be 16-byte aligned");
 

@@ -300,7 +300,7 @@ SP_DEVINL void epilogue_tma(const GemmEpi& e, const CUtensorMap* tmO, uint32_t t
                             bool live, int nb, uint8_t* boxes, int& nbox, const Fix& fx, int* err) {
   float v[32];
   if (EPI == EPI_F32 || EPI == EPI_F32_ACC) {
-    const bool scaled = EPI == EPI_F32 && e.row_scale != nullptr;
+    const bool scaled = EPI == EPI_F32 && BN != 32 && e.row_scale != nullptr;
     const float rs = scaled && live ? __ldg(e.row_scale + row0 + lane) : 0.f;
 #pragma unroll 1
     for (int c = 0; c < BN / 32; ++c) {
@@ -632,7 +632,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (one thread)
     if (lane == 0) {
-      const uint32_t IDESC = EPI == EPI_F32 && args.e.row_scale ? umma_idesc_f16_f32(BM, BN) : umma_idesc_bf16_f32(BM, BN);
+      const uint32_t IDESC =
+          EPI == EPI_F32 && BN != 32 && args.e.row_scale ? umma_idesc_f16_f32(BM, BN) : umma_idesc_bf16_f32(BM, BN);
       int s = 0;
       uint32_t ph = 0;
       int it = 0;
