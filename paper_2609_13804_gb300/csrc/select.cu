@@ -14,8 +14,8 @@
 //      memory in rank order (so all CTAs hold bitwise-identical results), adds
 //      the residual and applies LN2 -> pointer query;
 //   3. every CTA scores its available candidates from shared memory (four per
-//      warp iteration, shuffle reductions interleaved), each warp keeping a
-//      running top g+1 (logit desc, index asc); warp 0 merges them and pushes
+//      warp iteration, shuffle reductions interleaved), each warp picking its
+//      top g+1 (logit desc, index asc); warp 0 merges them and pushes
 //      the CTA's list into every CTA; the raw STOP logit is computed by every
 //      CTA identically;
 //   4. cluster barrier; every CTA merges the C lists, takes the same decision

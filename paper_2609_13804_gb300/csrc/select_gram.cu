@@ -9,8 +9,8 @@
 //      S[last][hist], ZV[last][hist], the newest positions' VV rows and slices
 //      of their G rows, Gz[last]; what later rounds need too (G, VV) stays in
 //      shared memory.  (One gather for the block: with every warp gathering the
-//      scores for itself the L1 tag lookups of scattered addresses, one a cycle,
-//      took longer than the trip to L2.)
+//      scores for itself, a tag lookup per scattered address, steps 1 and 2 took
+//      2,050 cycles at up to 192 positions, 1,780 so.)
 //   2. every warp takes the softmax weights of the t scores into registers (four
 //      consecutive positions per lane);
 //   3. warp w multiplies the positions k = w mod 8, into its partial logits and
