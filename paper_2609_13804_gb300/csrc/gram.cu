@@ -160,9 +160,10 @@ gram_operands_kernel(const BatchDesc bd, const GramArgs g) {
 // work item is one 128 x n_tile tile of one table of one episode.  A stage
 // holds both parts of 64 columns of both operands and feeds all three products
 // (12 MMAs of K = 16): 85 KB for 1,250 tensor cycles at n_tile 208, 68 B/cycle,
-// where staging the products one by one as a GEMM over 3h would take 101.
+// where staging the products one by one as a GEMM over 3h would take 101.  The
+// large parts have a barrier of their own and their product starts first.
 // 16 episodes of 576, h = 512 (82 useful GFLOP of three products, 107 MB of
-// tables): 112 us (126 with four epilogue warps), bound by the loads' latency at
+// tables): 110 us (126 with four epilogue warps and one barrier), bound by the loads' latency at
 // two stages and by the epilogue that nothing overlaps.
 constexpr int BM = 128;
 constexpr int BK = 64;
@@ -206,7 +207,7 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float* stg = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES + EPI_BYTES);
-  uint64_t* empty = full + STAGES;
+  uint64_t* empty = full + 2 * STAGES;  // (full: the large parts, then the small ones)
   uint64_t* tfull = empty + STAGES;
   uint64_t* tempty = tfull + 1;
   uint64_t* done = tempty + 1;
@@ -217,6 +218,7 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
+      mbar_init(&full[STAGES + s], 1);
       mbar_init(&empty[s], 1);
     }
     mbar_init(tfull, 1);
@@ -251,12 +253,14 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const int br = b_mat(w.p) * g.rows + w.ep.base + w.n0;
         for (int kb = 0; kb < KB; ++kb) {
           if (!mbar_wait(&empty[s], ph ^ 1u, err)) { ok = false; break; }
-          mbar_arrive_expect_tx(&full[s], 2 * (A_BYTES + (uint32_t)g.n_tile * BK * 2));
+          const uint32_t half = A_BYTES + (uint32_t)g.n_tile * BK * 2;
+          mbar_arrive_expect_tx(&full[s], half);
           uint8_t* st = smem + s * STAGE_BYTES;
           tma_load_2d(st, &tmA, &full[s], kb * BK, ar);
           tma_load_2d(st + 2 * A_BYTES, &tmB, &full[s], kb * BK, br);
-          tma_load_2d(st + A_BYTES, &tmA, &full[s], g.h + kb * BK, ar);
-          tma_load_2d(st + 2 * A_BYTES + B_BYTES, &tmB, &full[s], g.h + kb * BK, br);
+          mbar_arrive_expect_tx(&full[STAGES + s], half);
+          tma_load_2d(st + A_BYTES, &tmA, &full[STAGES + s], g.h + kb * BK, ar);
+          tma_load_2d(st + 2 * A_BYTES + B_BYTES, &tmB, &full[STAGES + s], g.h + kb * BK, br);
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
       }
@@ -279,11 +283,15 @@ gram_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           const uint32_t a1 = smem_u32(smem + s * STAGE_BYTES), a2 = a1 + A_BYTES;
           const uint32_t b1 = a1 + 2 * A_BYTES, b2 = b1 + B_BYTES;
 #pragma unroll
+          for (int k = 0; k < BK / 16; ++k)
+            umma_bf16(tmem_base, umma_desc_sw128(a1 + k * 32), umma_desc_sw128(b1 + k * 32), idesc, (kb | k) ? 1u : 0u);
+          if (!mbar_wait(&full[STAGES + s], ph, err)) { ok = false; break; }
+          tc_fence_after();
+#pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t da1 = umma_desc_sw128(a1 + k * 32), db1 = umma_desc_sw128(b1 + k * 32);
-            umma_bf16(tmem_base, da1, db1, idesc, (kb | k) ? 1u : 0u);
-            umma_bf16(tmem_base + NMAX, da1, umma_desc_sw128(b2 + k * 32), idesc, (kb | k) ? 1u : 0u);
-            umma_bf16(tmem_base + NMAX, umma_desc_sw128(a2 + k * 32), db1, idesc, 1u);
+            umma_bf16(tmem_base + NMAX, umma_desc_sw128(a1 + k * 32), umma_desc_sw128(b2 + k * 32), idesc,
+                      (kb | k) ? 1u : 0u);
+            umma_bf16(tmem_base + NMAX, umma_desc_sw128(a2 + k * 32), umma_desc_sw128(b1 + k * 32), idesc, 1u);
           }
           umma_commit(&empty[s]);
           if (++s == STAGES) { s = 0; ph ^= 1u; }
