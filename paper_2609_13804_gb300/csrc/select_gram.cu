@@ -21,7 +21,8 @@
 //      applies rstd and the LN2 bias term.  g = 1: the logit goes to every CTA of
 //      the cluster; grouped rounds: each warp's top g+1 does;
 //   5. the CTA waits for all n logits (they count their bytes on its mbarrier; no
-//      cluster barrier and no fence) and finds the best, or, grouped, every warp
+//      cluster barrier and no fence; a CTA without candidates sends one word, so
+//      that nobody runs ahead of it) and finds the best, or, grouped, every warp
 //      merges the lists after a cluster barrier; it takes the decision itself:
 //      nothing else is exchanged.
 // Three block barriers, one exchange and one trip to L2 per round, where the
@@ -38,6 +39,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "select_common.cuh"
+#include "select_slices.h"
 
 namespace cg = cooperative_groups;
 
@@ -141,9 +143,9 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
   const int n = min(gs, n_img - c0);
   const int row0 = bd.vis_off[lo] + c0;
   const int base = row0 + 2 * e;  // operand row of candidate 0
-  const int n_loc = (n + C - 1) / C;
-  const int j0 = rank * n_loc;
-  const int nl = max(0, min(j0 + n_loc, n) - j0);
+  const Slice slice = slice_of(n, C, rank);
+  const int j0 = slice.j0, nl = slice.nl;
+  const int round_bytes = 4 * words_of_round(n, C);
   const int lc = up4(n_loc_max + 1);
   const int wl = (n_loc_max + 31) >> 5;  // warps (lists) per CTA
   const int lists = C * wl;
@@ -156,7 +158,7 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
   float4* qp = reinterpret_cast<float4*>(sm + L.qp);
   float* sc_s = reinterpret_cast<float*>(sm + L.sc);
   float* zv_s = reinterpret_cast<float*>(sm + L.zv);
-  uint32_t* all_key = reinterpret_cast<uint32_t*>(sm + L.key);  // [parity][candidate], 0: taken
+  uint32_t* all_key = reinterpret_cast<uint32_t*>(sm + L.key);  // [parity][C * n_loc_max]: candidates' keys, 0: taken
   float* all_tv = reinterpret_cast<float*>(sm + L.tv);
   int* all_ti = reinterpret_cast<int*>(sm + L.ti);
   float* stop_s = reinterpret_cast<float*>(sm + L.misc);
@@ -249,8 +251,8 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
       sc_s[tid] = is_pos ? sc : -INFINITY;
       zv_s[tid] = zv;
     }
-    // the keys of all n candidates arrive on this round's barrier
-    if (GL == 2 && tid == 0) mbar_arrive_expect_tx(&mbar[buf], 4u * (uint32_t)n);
+    // the words of every CTA, the keys of all n candidates among them, arrive on this round's barrier
+    if (GL == 2 && tid == 0) mbar_arrive_expect_tx(&mbar[buf], (uint32_t)round_bytes);
 #pragma unroll
     for (int q = 0; q < NG; ++q) {
       const int k = t0 + q;
@@ -336,9 +338,9 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
         if (tid == nl) stop_s[buf] = v;
       }
       if (GL == 2) {
-        if (tid < nl) {
+        if (tid < slice.words) {
           const uint32_t key = avail ? fkey(v) : 0u;
-          const uint32_t d = smem_u32(all_key + buf * n_keys + col), mb = smem_u32(&mbar[buf]);
+          const uint32_t d = smem_u32(all_key + buf * n_keys + j0 + tid), mb = smem_u32(&mbar[buf]);
 #pragma unroll
           for (int r = 0; r < kMaxCluster; ++r)
             if (r < C) st_async_u32(mapa_shared(d, r), key, mapa_shared(mb, r));

@@ -51,6 +51,7 @@ def test_encoder_row_forms(B, D):
 
 @pytest.mark.parametrize("n_vis,h,g,k_max,group", [
     ([1, 126, 2, 127], 128, 1, 8, 0),          # one row tile, its last row and one more
+    ([1, 9, 17, 33, 49], 128, 1, 49, 0),       # CTAs without candidates
     ([254, 255, 31], 256, 1, 40, 0),           # the edges of one column tile
     ([509, 33], 512, 1, 96, 0),                # history registers at their smaller capacity
     ([330], 1024, 1, 223, 0),                  # and at the larger one
