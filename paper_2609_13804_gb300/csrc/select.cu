@@ -387,7 +387,7 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
   const float bias = __ldg(a.stop_bias + e);
   const size_t trace = (size_t)e * (k_max + 1);
   tc_fence_before();
-  __syncthreads();
+  cluster.sync();  // (every CTA has started before the first push into its shared memory)
   tc_fence_after();
   const int ppw = tm_cols / (16 * HV);  // cached positions per warp
   const uint32_t tm_base = tm_cols > 0 ? *tm_slot : 0u;

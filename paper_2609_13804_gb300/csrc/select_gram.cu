@@ -207,8 +207,8 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
       mbar_init(&mbar[1], 1);
       fence_mbar_init();
     }
-    cluster.sync();  // every CTA's barriers are ready before the first push
   }
+  cluster.sync();  // every CTA has started, and its barriers are ready, before the first push
 
   int hist = n + 1;  // index of history position tid (START at 0)
   int hnew[NG];      // positions that joined last
