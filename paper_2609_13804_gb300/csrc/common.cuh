@@ -172,6 +172,7 @@ SP_DEVINL bool wait_flag(const int* flag, int* err, uint64_t limit_ns = kWaitLim
 SP_DEVINL bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err) {
   bool ok = true;
   if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, err);
+  __syncwarp();  // (orders the other lanes' reads behind lane 0's acquire: a shuffle does not)
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
@@ -520,6 +521,7 @@ SP_DEVINL bool mbar_wait_cluster_warp(uint64_t* bar, uint32_t parity, int* err) 
       }
     }
   }
+  __syncwarp();  // (orders the other lanes' reads behind lane 0's acquire: a shuffle does not)
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 

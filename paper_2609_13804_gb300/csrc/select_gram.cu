@@ -115,6 +115,7 @@ SP_DEVINL bool mbar_poll_cluster_warp(uint64_t* bar, uint32_t parity, int* err) 
       }
     }
   }
+  __syncwarp();  // (orders the other lanes' reads behind lane 0's acquire: a shuffle does not)
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
