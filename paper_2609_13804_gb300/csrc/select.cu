@@ -1315,7 +1315,9 @@ cudaError_t select_launch(const BatchDesc& bd, int n_episodes, const SelectArgs&
     default: return cudaErrorInvalidValue;
   }
 #undef SP_SEL_CASE
-  cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
+  // (one limit whatever the size: another thread may set it between this call and the launch)
+  if (L.total > kSmemBudget) return cudaErrorInvalidValue;
+  cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
   if (r != cudaSuccess) return r;
   if (C > 8) {
     r = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

@@ -530,7 +530,8 @@ cudaError_t select_gram_launch(const BatchDesc& bd, int n_episodes, const Select
                : (gl == 2 ? select_gram_kernel<2, false>
                           : (gl == 6 ? select_gram_kernel<6, false> : select_gram_kernel<17, false>));
   if (T > kMaxHist || C > kMaxCluster) return cudaErrorInvalidValue;
-  cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (one limit whatever the size: another thread may set it between this call and the launch)
+  cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
   if (r != cudaSuccess) return r;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_episodes * C, 1, 1);

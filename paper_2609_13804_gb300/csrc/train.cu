@@ -143,7 +143,9 @@ cudaError_t soft_topk_launch(const BatchDesc& bd, int n_episodes, const float* s
   for (int b = 0; b < bd.B; ++b) n_max = std::max(n_max, bd.vis_off[b + 1] - bd.vis_off[b]);
   const size_t smem = (size_t)std::max(n_max, 1) * sizeof(float);
   if (smem > 48 * 1024) {
-    cudaError_t r = cudaFuncSetAttribute(soft_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (one limit whatever the size: another thread may set it between this call and the launch)
+    cudaError_t r = cudaFuncSetAttribute(soft_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(SP_MAX_NVIS * sizeof(float)));
     if (r != cudaSuccess) return r;
   }
   prof_begin_launch(st);

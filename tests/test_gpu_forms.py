@@ -1,4 +1,6 @@
 """The forms that a dispatch rule chooses between by size, at the edges of their ranges."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -24,6 +26,12 @@ def B():
 
 def np_(t):
     return t.float().cpu().numpy() if t.dtype == torch.bfloat16 else t.cpu().numpy()
+
+
+def general_workspace(n_vis, D, h):
+    """What the general kernel carves from a given memory (one layer, D >= h), in 256-byte slices."""
+    rows = sum(n_vis) + 2
+    return 4 * rows * (D + h + 2 * h + 3 * h) + 2 * rows * 3 * D + 4 * len(n_vis) * 1024 + 16 * 256
 
 
 @pytest.mark.parametrize("D", [384, 2176, 4096, 4224])
@@ -72,8 +80,7 @@ def test_selection_tables_and_keys_agree(B):
     selector = B.Selector(s, PT.scale_decoder(S.make_selector_weights(w, ln_affine=True), 4.0), DEV)
     H, bias = B.dev_f32(S.make_memory(w), DEV), B.dev_f32(np.full(2, -1e30, np.float32), DEV)
     full = B.sp_select(selector, w.n_vis, w.n_txt, H=H, stop_bias=bias, k_max=48)
-    rows = sum(w.n_vis) + 2  # what the general kernel carves, 256-byte slices
-    need = 4 * rows * (128 + 128 + 2 * 128 + 3 * 128) + 2 * rows * 3 * 128 + 4 * 2 * 1024 + 16 * 256
+    need = general_workspace(w.n_vis, 128, 128)
     assert need < full["_ws"].numel()
     small = B.sp_select(selector, w.n_vis, w.n_txt, H=H, stop_bias=bias, k_max=48, ws=full["_ws"][:need].clone())
     torch.cuda.synchronize()
@@ -82,4 +89,38 @@ def test_selection_tables_and_keys_agree(B):
     np.testing.assert_array_equal(np_(full["order"]), np_(small["order"]))
     g0, g1 = np_(full["gap"])[:, :48], np_(small["gap"])[:, :48]
     assert np.abs(g0 - g1).max() <= 2e-4 * max(1.0, np.abs(g1).max())
+    selector.close()
+
+
+def test_selections_of_different_sizes_from_two_threads(B):
+    """Every selection gets the shared memory that its own size needs, whatever another thread launches meanwhile.
+    (STOP wins at once, so that the threads spend their time launching.)"""
+    shapes = [([24, 24], 8), ([1016, 900], 223)]
+    w = [S.tiny_workload(96 + i, n, [1, 1], D=128, D_text=128, h=128, k_max=k) for i, (n, k) in enumerate(shapes)]
+    s = S.SelectorShape(D=128, D_text=128, h=128, n_enc_layers=0)
+    selector = B.Selector(s, S.make_selector_weights(w[0]), DEV)
+    bias = B.dev_f32(np.full(2, 1e30, np.float32), DEV)
+    H = [B.dev_f32(S.make_memory(x), DEV) for x in w]
+    failed = []
+
+    def work(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                ws = None
+                for _ in range(3000):
+                    out = B.sp_select(selector, w[i].n_vis, w[i].n_txt, H=H[i], stop_bias=bias, k_max=w[i].k_max,
+                                      traces=False, ws=ws)
+                    ws = out["_ws"]
+                torch.cuda.current_stream().synchronize()
+            assert int(out["err"].item()) == 0 and out["count"].tolist() == [0, 0]
+        except Exception as e:
+            failed.append((shapes[i], e))
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
     selector.close()
