@@ -119,8 +119,63 @@ SP_DEVINL bool mbar_poll_cluster_warp(uint64_t* bar, uint32_t parity, int* err) 
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
+// LN2's variance from the tables is a sum of products of either sign. Where the
+// residual and the attention output, or the values among themselves, cancel, its
+// rounding grows with the square of the cancellation, that of the formed vector
+// only with its first power. In the careful form of the rounds the vector is
+// formed where the variance is below 1 / kCancel of what its terms come to
+// without the cross terms (rows independent of one another: near 1; at 1 / 8 the
+// tables' variance is still good to 3e-6). The usual form is for episodes where
+// that cannot happen: no value longer than half of any residual (the ratio stays
+// above 0.2), and START by itself no cancellation. Each form is a kernel, and
+// both are launched: the usual one asks the question as it starts and leaves its
+// answer in the table for the other. (Asked in every round it costs 2 to 5 % of
+// the rounds, and with both forms in one kernel the usual one was 15 % slower;
+// the question and the second launch are 2 to 5 us a call.)
+constexpr float kCancel = 8.f;
+
+// |zc_last + sum_k p_k vc_k|^2 from the operand rows of the tables (their fp16
+// parts sum to the fp32 row up to 2^-23), all threads of the block: t rows of
+// 4 h bytes from L2 by every CTA, in place of a few adds.  p_k = exp(sc_s[k] -
+// mx) inv_sum; hist_s: the positions' rows, not yet synchronised; red: NW floats.
+__device__ __noinline__ float direct_variance(const __half2* op, const float* inv, int rows, int base, int h, int last,
+                                              int t, const float* sc_s, float mx, float inv_sum, const int* hist_s,
+                                              float* red) {
+  __syncthreads();
+  const int h2 = h >> 1;
+  auto row_of = [&](int m, int i) { return op + ((size_t)m * rows + base + i) * h; };
+  auto at = [&](const __half2* r, int c) {
+    const float2 a = __half22float2(r[c]), b = __half22float2(r[h2 + c]);
+    return make_float2(a.x + b.x, a.y + b.y);
+  };
+  float s = 0.f;
+  for (int c = threadIdx.x; c < h2; c += NT) {
+    float2 o = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int k = 0; k < t; ++k) {
+      const int i = hist_s[k];
+      const float p = __expf(sc_s[k] - mx) * inv[2 * rows + base + i];
+      const float2 v = at(row_of(2, i), c);
+      o.x = fmaf(p, v.x, o.x);
+      o.y = fmaf(p, v.y, o.y);
+    }
+    const float iz = inv[3 * rows + base + last];
+    const float2 z = at(row_of(3, last), c);
+    const float x = fmaf(z.x, iz, o.x * inv_sum), y = fmaf(z.y, iz, o.y * inv_sum);
+    s = fmaf(x, x, fmaf(y, y, s));
+  }
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = 0.f;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) s += red[w];
+  __syncthreads();
+  return s;
+}
+
 // GL: capacity of the top lists (g + 1 <= GL).
-template <int GL, bool TRAIN>
+template <int GL, bool TRAIN, bool CAREFUL>
 __global__ void __launch_bounds__(NT, 1)
 select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, int n_loc_max, int T_max) {
   constexpr int NG = GL - 1;  // new positions per round at most
@@ -151,6 +206,11 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
   const int wl = (n_loc_max + 31) >> 5;  // warps (lists) per CTA
   const int lists = C * wl;
 
+  float* tab = gr.table + (size_t)e * gr.ep_stride;
+  const int ld = gr.ld;
+  float* flag = tab + (size_t)n * (5 * ld);  // (STOP is never in the history: its row is free)
+  if (CAREFUL && *flag == 0.f) return;
+
   extern __shared__ __align__(16) uint8_t sm[];
   const GramSmem L = gram_smem(T_max, n_loc_max, C, per);
   float* Gs = reinterpret_cast<float*>(sm + L.G);
@@ -166,8 +226,6 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + L.misc + 16);
   uint4* best_s = reinterpret_cast<uint4*>(sm + L.misc + 32);  // per warp: key, index, softmax sum
 
-  const float* tab = gr.table + (size_t)e * gr.ep_stride;
-  const int ld = gr.ld;
   const float bias = __ldg(a.stop_bias + e);
   const size_t trace = (size_t)e * (k_max + 1);
   const bool tracer = rank == 0 && tid == NT - 32;    // writes the traces, in a warp without a candidate list
@@ -202,6 +260,20 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
   float tr_best = 0.f, tr_raw = 0.f;
   int tr_j = -1, tr_round = 0, tr_nsel = 0;  // (-1: no round to trace)
 
+  float vmax = 0.f, zmin = INFINITY, z2 = 0.f, zv2 = 0.f, v2 = 0.f;  // squared lengths; START's products
+  if (!CAREFUL) {
+    const float* start = tab + (size_t)(n + 1) * (5 * ld) + n + 1;
+    z2 = gr.zz[base + n + 1];
+    v2 = start[3 * ld];
+    zv2 = start[4 * ld];
+    for (int i = tid; i < n; i += NT) {
+      vmax = fmaxf(vmax, tab[(size_t)i * (5 * ld) + 3 * ld + i]);
+      zmin = fminf(zmin, gr.zz[base + i]);
+    }
+    vmax = warp_max(vmax);
+    zmin = -warp_max(-zmin);
+    if (lane == 0) qp[warp] = make_float4(vmax, zmin, 0.f, 0.f);
+  }
   if (GL == 2) {
     if (tid == 0) {
       mbar_init(&mbar[0], 1);
@@ -210,6 +282,18 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
     }
   }
   cluster.sync();  // every CTA has started, and its barriers are ready, before the first push
+
+  if (!CAREFUL) {
+    vmax = v2;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      vmax = fmaxf(vmax, qp[w].x);
+      zmin = fminf(zmin, qp[w].y);
+    }
+    const bool careful = 4.f * vmax > zmin || kCancel * (z2 + 2.f * zv2 + v2) < z2 + v2;  // (the same in every CTA)
+    if (rank == 0 && tid == 0) *flag = careful ? 1.f : 0.f;
+    if (careful) return;
+  }
 
   int hist = n + 1;  // index of history position tid (START at 0)
   int hnew[NG];      // positions that joined last
@@ -284,6 +368,12 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
       if (i1 < t) dot(p1, 32 + lane);
     }
 
+    float own = 0.f;  // this thread's position by itself
+    if (CAREFUL && is_pos) {
+      const float p = __expf(sc - mx);
+      own = p * p * vvs[vv_row(tid) + tid];
+    }
+
     // ---- 3. this warp's positions
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     float quad = 0.f, sum = 0.f;
@@ -312,13 +402,33 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
     for (int o = 16; o > 0; o >>= 1) {
       quad += __shfl_xor_sync(0xffffffffu, quad, o);
       lin += __shfl_xor_sync(0xffffffffu, lin, o);
+      if (CAREFUL) own += __shfl_xor_sync(0xffffffffu, own, o);
     }
-    if (lane == 0) qp[warp] = make_float4(sum, lin, quad, 0.f);
+    if (lane == 0) qp[warp] = make_float4(sum, lin, quad, own);
     if (i0 <= nl) *reinterpret_cast<float4*>(lgp + warp * lc + i0) = acc;
     __syncthreads();
 
     // ---- 4. logits, exchange
     float v = -INFINITY;
+    float formed = -1.f;
+    if (CAREFUL) {
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const float4 y = qp[w];
+        x.x += y.x;
+        x.y += y.y;
+        x.z += y.z;
+        x.w += y.w;
+      }
+      const float inv = 1.f / x.x;
+      if (kCancel * (zz + inv * (2.f * x.y + inv * x.z)) < zz + inv * inv * x.w) {  // (the same in every CTA)
+        int* hist_s = reinterpret_cast<int*>(zv_s);
+        if (is_pos) hist_s[tid] = hist;
+        formed = direct_variance(static_cast<const __half2*>(gr.op), gr.inv, gr.rows, base, a.h, last, t, sc_s, mx, inv,
+                                 hist_s, reinterpret_cast<float*>(best_s));
+      }
+    }
     if (warp <= (n_loc_max >> 5)) {  // (threads 0 .. nl)
       float ps = 0.f, pl = 0.f, pq = 0.f;
 #pragma unroll
@@ -329,7 +439,7 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
         pq += x.z;
       }
       const float inv = 1.f / ps;
-      const float var = zz + inv * (2.f * pl + inv * pq);
+      const float var = CAREFUL && formed >= 0.f ? formed : zz + inv * (2.f * pl + inv * pq);
       const float rstd = rsqrtf(fmaxf(var * inv_h, 0.f) + a.ln_eps);
       if (is_col) {
         float x = 0.f;
@@ -516,27 +626,21 @@ int select_gram_cluster(int n_max, int k_max, int g) {
   return 0;
 }
 
-cudaError_t select_gram_launch(const BatchDesc& bd, int n_episodes, const SelectArgs& a, const GramArgs& g, int n_max,
-                               int C, cudaStream_t st) {
-  if (n_episodes <= 0) return cudaSuccess;
-  const int n_loc = (n_max + C - 1) / C;
-  const int T = gram_history(a.k_max, n_max);
-  const size_t smem = gram_smem(T, n_loc, C, a.g + 1).total;
-  const int gl = a.g + 1 <= 2 ? 2 : (a.g + 1 <= 6 ? 6 : 17);
-  const bool train = a.score != nullptr;
-  if (train && (a.g != 1 || !a.kbar)) return cudaErrorInvalidValue;
-  void (*kern)(const BatchDesc, const SelectArgs, const GramArgs, int, int) = nullptr;
-  kern = train ? select_gram_kernel<2, true>
-               : (gl == 2 ? select_gram_kernel<2, false>
-                          : (gl == 6 ? select_gram_kernel<6, false> : select_gram_kernel<17, false>));
-  if (T > kMaxHist || C > kMaxCluster) return cudaErrorInvalidValue;
+template <bool CAREFUL>
+static cudaError_t launch_form(const BatchDesc& bd, int n_episodes, const SelectArgs& a, const GramArgs& g, int n_loc,
+                               int T, int C, cudaStream_t st) {
+  const int per = a.g + 1;
+  void (*kern)(const BatchDesc, const SelectArgs, const GramArgs, int, int) =
+      a.score ? select_gram_kernel<2, true, CAREFUL>
+              : (per <= 2 ? select_gram_kernel<2, false, CAREFUL>
+                          : (per <= 6 ? select_gram_kernel<6, false, CAREFUL> : select_gram_kernel<17, false, CAREFUL>));
   // (one limit whatever the size: another thread may set it between this call and the launch)
   cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
   if (r != cudaSuccess) return r;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_episodes * C, 1, 1);
   cfg.blockDim = dim3(NT, 1, 1);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = gram_smem(T, n_loc, C, per).total;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -551,6 +655,18 @@ cudaError_t select_gram_launch(const BatchDesc& bd, int n_episodes, const Select
   r = cudaLaunchKernelEx(&cfg, kern, bd, a, g, n_loc, T);
   prof_end_launch(st, SP_K_SELECT, 0.0, 0.0);
   return r;
+}
+
+cudaError_t select_gram_launch(const BatchDesc& bd, int n_episodes, const SelectArgs& a, const GramArgs& g, int n_max,
+                               int C, cudaStream_t st) {
+  if (n_episodes <= 0) return cudaSuccess;
+  const int n_loc = (n_max + C - 1) / C;
+  const int T = gram_history(a.k_max, n_max);
+  const bool train = a.score != nullptr;
+  if (train && (a.g != 1 || !a.kbar)) return cudaErrorInvalidValue;
+  if (T > kMaxHist || C > kMaxCluster) return cudaErrorInvalidValue;
+  const cudaError_t r = launch_form<false>(bd, n_episodes, a, g, n_loc, T, C, st);
+  return r == cudaSuccess ? launch_form<true>(bd, n_episodes, a, g, n_loc, T, C, st) : r;
 }
 
 }  // namespace sp

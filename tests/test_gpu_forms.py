@@ -8,6 +8,7 @@ from oracle import core as O
 from paper_2609_13804_gb300 import synth as S
 import _parity as PT
 import test_gpu_parity as GP
+import test_gpu_train as GT
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -57,6 +58,26 @@ def test_encoder_row_forms(B, D):
     selector.close()
 
 
+def attention_can_cancel(H, sel):
+    """Whether the tables' kernel asks in its rounds for a cancelling attention output (none of these decoders'
+    START rows cancels by itself): a value longer than half of a residual."""
+    z = O.decoder_tokens(np.concatenate([H, sel["s_start"][None]]).astype(np.float64), sel)
+    x = O.layer_norm(z, 1e-5, sel.get("ln1_g"), sel.get("ln1_b"))
+    v = x @ sel["Wv_s"].T.astype(np.float64) @ sel["Wo_s"].T.astype(np.float64)
+    z, v = z - z.mean(-1, keepdims=True), v - v.mean(-1, keepdims=True)
+    return 4 * (v ** 2).sum(-1).max() > (z[:-1] ** 2).sum(-1).min()
+
+
+def run_with_tables(B, run):
+    """run(), which makes one selection: by tables, whose two kernels are launched together."""
+    B.sp_profile_begin()
+    try:
+        return run()
+    finally:
+        assert B.sp_profile_end()["select"]["launches"] == 2
+
+
+@pytest.mark.parametrize("D", [128, 1024])     # attention outputs that may cancel the residual, and that cannot
 @pytest.mark.parametrize("n_vis,h,g,k_max,group", [
     ([1, 126, 2, 127], 128, 1, 8, 0),          # one row tile, its last row and one more
     ([1, 9, 17, 33, 49], 128, 1, 49, 0),       # CTAs without candidates
@@ -66,11 +87,24 @@ def test_encoder_row_forms(B, D):
     ([1016, 700], 128, 5, 120, 0),             # the widest slices, grouped rounds
     ([64, 300], 128, 16, 100, 100),            # candidate groups, the longest lists
 ])
-def test_selection_tables(B, n_vis, h, g, k_max, group):
+def test_selection_tables(B, n_vis, h, g, k_max, group, D):
     """The table-driven selection at the edges of its tiles, slices and lists, with LN2's gain and bias."""
-    w = S.tiny_workload(93, n_vis, [1] * len(n_vis), D=128, D_text=128, h=h, enc_head_dim=64, k_max=k_max,
+    w = S.tiny_workload(93, n_vis, [1] * len(n_vis), D=D, D_text=128, h=h, enc_head_dim=64, k_max=k_max,
                         group_size=group, g=g)
-    GP._run_select_case(B, w, scale=4.0 if h <= 256 else 2.0)
+    scale = (4.0 if h <= 256 else 2.0) if D == 128 else min(3.0, 512.0 / h)
+    sel = PT.scale_decoder(S.make_selector_weights(w, ln_affine=True), scale)
+    assert attention_can_cancel(S.make_memory(w), sel) == (D == 128)
+    run_with_tables(B, lambda: GP._run_select_case(B, w, scale=scale))
+
+
+@pytest.mark.parametrize("D", [128, 1024])
+def test_training_tables(B, D):
+    """The aggregates from the tables over a long history, in both forms of the rounds."""
+    w = S.tiny_workload(94, [260, 210], [1, 1], D=D, D_text=128, h=128, k_max=200)
+    scale = 4.0 if D == 128 else 3.0
+    sel = PT.scale_decoder(S.make_selector_weights(w, ln_affine=True), scale)
+    assert attention_can_cancel(S.make_memory(w), sel) == (D == 128)
+    GT._train_case(B, w, tau=1.0, beta=0.99, scale=scale, targets=[200, 150])
 
 
 def test_selection_tables_and_keys_agree(B):
@@ -79,7 +113,7 @@ def test_selection_tables_and_keys_agree(B):
     s = S.SelectorShape(D=128, D_text=128, h=128, n_enc_layers=0)
     selector = B.Selector(s, PT.scale_decoder(S.make_selector_weights(w, ln_affine=True), 4.0), DEV)
     H, bias = B.dev_f32(S.make_memory(w), DEV), B.dev_f32(np.full(2, -1e30, np.float32), DEV)
-    full = B.sp_select(selector, w.n_vis, w.n_txt, H=H, stop_bias=bias, k_max=48)
+    full = run_with_tables(B, lambda: B.sp_select(selector, w.n_vis, w.n_txt, H=H, stop_bias=bias, k_max=48))
     need = general_workspace(w.n_vis, 128, 128)
     assert need < full["_ws"].numel()
     small = B.sp_select(selector, w.n_vis, w.n_txt, H=H, stop_bias=bias, k_max=48, ws=full["_ws"][:need].clone())
@@ -123,4 +157,39 @@ def test_selections_of_different_sizes_from_two_threads(B):
     for t in threads:
         t.join()
     assert not failed, failed
+    selector.close()
+
+
+def test_selection_tables_where_attention_cancels_the_residual(B):
+    """A decoder whose attention output is nearly the negative of its residual (|u| about 0.03 |z|): the tables'
+    logits are as close to the 64-bit ones as the general kernel's, which forms u.  Both start from the same
+    precomputed rows, whose rounding that cancellation magnifies alike."""
+    n, h, k = [300], 128, 24
+    w = S.tiny_workload(97, n, [1], D=128, D_text=128, h=h, k_max=k)
+    sel = PT.scale_decoder(S.make_selector_weights(w, ln_affine=False), 4.0)
+    eye = np.eye(h, dtype=np.float32)
+    sel["Wq_s"], sel["Wk_s"] = 1.5 * eye, 1.5 * eye  # every position attends to itself
+    sel["Wv_s"], sel["Wo_s"] = eye, (-0.98 * eye + 0.02 / np.sqrt(h) * S.normal(97, "R", (h, h))).astype(np.float32)
+
+    def unit(m):  # decoder tokens with a standard deviation of one
+        return (m / (m.astype(np.float64) @ sel["W_in"].T.astype(np.float64)).std(-1, keepdims=True)).astype(np.float32)
+
+    H, sel["s_start"] = unit(S.make_memory(w)), unit(sel["s_start"][None])[0]
+    bias = np.full(1, -1e30, np.float32)
+    selector = B.Selector(S.SelectorShape(D=128, D_text=128, h=h, n_enc_layers=0), sel, DEV)
+    args = dict(H=B.dev_f32(H, DEV), stop_bias=B.dev_f32(bias, DEV), k_max=k)
+    full = run_with_tables(B, lambda: B.sp_select(selector, n, [1], **args))
+    need = general_workspace(n, 128, h)
+    assert need < full["_ws"].numel()
+    small = B.sp_select(selector, n, [1], ws=full["_ws"][:need].clone(), **args)
+    torch.cuda.synchronize()
+    replay, _ = PT.replayer(H, n, sel, k_max=k, g=1, group_size=0, biases=bias)
+    err = []
+    for out in (full, small):
+        assert int(out["err"].item()) == 0
+        ref = np.asarray(replay(0, [int(x) for x in np_(out["order"])[0]])["gap"][:k])
+        err.append(np.linalg.norm(np_(out["gap"])[0, :k] - ref) / np.linalg.norm(ref))
+    print("relative errors of the gaps, tables and general kernel:", err)
+    # (two roundings of the operands in place of one)
+    assert err[0] <= 2 * err[1], err
     selector.close()
