@@ -749,8 +749,12 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
   a.KC = ZK + 2 * h;
   a.dcache = static_cast<float*>(parts[15]);
   a.dcache_ep = (size_t)(s->n_dec - 1) * (in->k_max + 1) * 2 * h;
+  bool keys_smem = true;
+  size_t smem = 0;
+  const int C = select_cluster_size(p.bd, h, in->k_max, &keys_smem, &smem, s->n_dec > 1);
   if (p.gram_C) {
     GramArgs ga = p.gram;
+    ga.pass_nan = !keys_smem;
     ga.Z = a.Z; ga.ldz = a.ldz;
     ga.KT = a.KT; ga.ldkt = a.ldkt;
     ga.QS = a.QS; ga.ldqs = a.ldqs;
@@ -767,9 +771,6 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
     SP_CUDA(gram_launch(p.bd, ga, st), "selection tables");
     SP_CUDA(select_gram_launch(p.bd, p.E, a, ga, p.n_max, p.gram_C, st), "selection");
   } else {
-    bool keys_smem = true;
-    size_t smem = 0;
-    const int C = select_cluster_size(p.bd, h, in->k_max, &keys_smem, &smem, s->n_dec > 1);
     SP_CUDA(select_launch(p.bd, p.E, a, C, keys_smem, smem, st), "selection");
   }
   SP_CUDA(restore_launch(p.bd, a.order, a.ep_count, in->k_max, out->idx, out->k_cap, out->count, err, st), "restore");

@@ -267,6 +267,7 @@ struct GramArgs {
   const float* VT; int ldvt;
   const float* ln2_g; const float* ln2_b;
   int stop_row, start_row;
+  bool pass_nan;           // NaN logits are passed over (select_cluster_size)
   void* op;                // [5][rows][2h] fp16: two parts of KTg, KS, vc, zc, QS
   float* inv;              // [5][rows] inverse scales
   float* dj;               // [rows] <kt, ln2 bias>
@@ -281,6 +282,9 @@ int select_gram_cluster(int n_max, int k_max, int g);
 cudaError_t select_gram_launch(const BatchDesc& bd, int n_episodes, const SelectArgs& a, const GramArgs& g, int n_max,
                                int C, cudaStream_t st);
 
+// Cluster size of the general kernel and whether its keys fit shared memory.
+// Streamed keys pass over a candidate whose logit is NaN, keys in shared memory
+// give it a rank; the table-driven kernel does what this one would.
 int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_smem, size_t* smem_bytes,
                         bool multi = false);
 cudaError_t select_launch(const BatchDesc& bd, int n_episodes, const SelectArgs& a,

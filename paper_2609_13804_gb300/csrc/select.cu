@@ -1016,7 +1016,7 @@ select_kernel(const BatchDesc bd, const SelectArgs a, int n_loc_max, int keys_in
       for (int i = 0; i < SP_MAX_NVIS / 16 / NT; ++i) {
         const int j = tid + NT * i;
         const bool ok = j < nl && !taken[j];
-        key[i] = ok ? fkey(lgp[j]) : 0u;
+        key[i] = ok ? logit_key(lgp[j], true) : 0u;
         id[i] = ok ? j0 + j : INT_MAX;
       }
 #pragma unroll

@@ -12,6 +12,8 @@ SP_DEVINL uint32_t fkey(float v) {
   const uint32_t u = __float_as_uint(v + 0.0f);
   return (u >> 31) ? ~u : (u | 0x80000000u);
 }
+// The key of a logit; a NaN ranks next to zero (its sign is the compiler's), or (pass_nan) is passed over.
+SP_DEVINL uint32_t logit_key(float v, bool pass_nan) { return pass_nan && v != v ? 0u : fkey(v); }
 SP_DEVINL float fkey_inv(uint32_t k) {
   if (k == 0u) return -INFINITY;
   return __uint_as_float((k >> 31) ? (k & 0x7FFFFFFFu) : ~k);

@@ -450,7 +450,7 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
       }
       if (GL == 2) {
         if (tid < slice.words) {
-          const uint32_t key = avail ? fkey(v) : 0u;
+          const uint32_t key = avail ? logit_key(v, gr.pass_nan) : 0u;
           const uint32_t d = smem_u32(all_key + buf * n_keys + j0 + tid), mb = smem_u32(&mbar[buf]);
 #pragma unroll
           for (int r = 0; r < kMaxCluster; ++r)
@@ -458,7 +458,7 @@ select_gram_kernel(const BatchDesc bd, const SelectArgs a, const GramArgs gr, in
         }
       } else if (warp < wl) {
         int id = avail ? col : INT_MAX;
-        uint32_t key = avail ? fkey(v) : 0u;
+        uint32_t key = avail ? logit_key(v, gr.pass_nan) : 0u;
         float* dv = all_tv + (size_t)(buf * lists + rank * wl + warp) * per;
         int* di = all_ti + (size_t)(buf * lists + rank * wl + warp) * per;
         if (lane < C) {

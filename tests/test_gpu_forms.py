@@ -193,3 +193,26 @@ def test_selection_tables_where_attention_cancels_the_residual(B):
     # (two roundings of the operands in place of one)
     assert err[0] <= 2 * err[1], err
     selector.close()
+
+
+@pytest.mark.parametrize("n,h,g,k_max", [(2100, 128, 1, 12), (2100, 128, 5, 12), (300, 1024, 1, 40), (300, 1024, 5, 60)])
+def test_a_nan_candidate_is_passed_over_where_keys_are_streamed(B, n, h, g, k_max):
+    """Episodes whose keys do not fit shared memory select as if a candidate with a NaN row were not there, also
+    where the tables take their place (h = 1,024 here). (All logits negative: the keys rank a NaN next to zero.)"""
+    w = S.tiny_workload(98, [n], [1], D=128, D_text=128, h=h, k_max=k_max)
+    sel = PT.scale_decoder(S.make_selector_weights(w, ln_affine=True), 4.0 if h == 128 else 1.0)
+    sel["ln2_b"] = 3 * S.normal(98, "b", (h,))
+    away = sel["Wk_p"].T @ sel["Wq_p"] @ sel["ln2_b"]
+    H, bias = S.make_memory(w) - 8 * away / np.linalg.norm(away), B.dev_f32(np.full(1, -1e30, np.float32), DEV)
+    selector = B.Selector(S.SelectorShape(D=128, D_text=128, h=h, n_enc_layers=0), sel, DEV)
+    j = n // 3
+    args = dict(stop_bias=bias, k_max=w.k_max, g=g)
+    want = B.sp_select(selector, [n - 1], [1], H=B.dev_f32(np.delete(H, j, 0), DEV), **args)
+    H[j] = np.nan
+    got = B.sp_select(selector, [n], [1], H=B.dev_f32(H, DEV), **args)
+    torch.cuda.synchronize()
+    assert int(got["err"].item()) == 0 and int(want["err"].item()) == 0
+    order = np_(want["order"])
+    np.testing.assert_array_equal(np_(got["order"]), order + (order >= j))
+    np.testing.assert_array_equal(np_(got["gap"]), np_(want["gap"]))
+    selector.close()
