@@ -1253,13 +1253,48 @@ restore_kernel(const BatchDesc bd, const int* order, const int* ep_count,
 
 }  // namespace
 
-// Episodes that all run at once as 16-CTA clusters (one per GPC).  A round of a
-// decoder of several layers streams the lower layers' weights and cross-attention
-// rows from L2 through its cluster's SMs: with half the rows per CTA 4 episodes
-// of 576 take 42 us a round in place of 62 (the pushes of 16 bytes a lane and the
-// row batches of the functions above included).
-constexpr int kWideClusters = 8;
 constexpr size_t kSmemBudget = 225 * 1024;
+
+using SelectKernel = void (*)(const BatchDesc, const SelectArgs, int, int, int);
+
+static SelectKernel deep_kernel(int h) {
+  switch (h / 128) {
+    case 1: return select_kernel<1, 2, false, true>;
+    case 2: return select_kernel<2, 2, false, true>;
+    case 4: return select_kernel<4, 2, false, true>;
+    case 8: return select_kernel<8, 2, false, true>;
+    default: return nullptr;
+  }
+}
+
+// A decoder of several layers streams the lower layers' weights and
+// cross-attention rows from L2 through its cluster's SMs in every round, so
+// 16-CTA clusters are taken where all episodes run at once in them (32 rounds,
+// 4 episodes: 576 candidates with h = 256 996 us, 8 CTAs 1,032; h = 512 1,483
+// and 1,822; 120 with h = 1,024, keys streamed, 2,099 and 2,572, keys held;
+// h = 128 the same within 3 %).  How many that is depends on the card: 7 where
+// a GPC is short of SMs, and 8 episodes of 576, h = 512, then took two waves and
+// 2,926 us, 1,918 with 8 CTAs.
+static bool wide_clusters_fit(int n_ep, int h, size_t smem) {
+  const SelectKernel kern = deep_kernel(h);
+  if (!kern || n_ep * 16 > device_sm_count()) return false;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return false;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_ep * 16, 1, 1);
+  cfg.blockDim = dim3(NT, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 16;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int active = 0;
+  return cudaOccupancyMaxActiveClusters(&active, kern, &cfg) == cudaSuccess && active >= n_ep;
+}
 
 int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_smem, size_t* smem_bytes, bool multi) {
   int n_max = 0;
@@ -1267,19 +1302,22 @@ int select_cluster_size(const BatchDesc& bd, int h, int k_max, bool* keys_in_sme
     const int n = bd.vis_off[b + 1] - bd.vis_off[b];
     n_max = std::max(n_max, bd.group_size > 0 ? std::min(bd.group_size, n) : n);
   }
-  const int n_ep = bd.ep_off[bd.B];
-  for (int C : {8, 16}) {
-    if (C == 8 && multi && n_ep <= kWideClusters) continue;
+  auto keys_fit = [&](int C) {
     const int n_loc = (n_max + C - 1) / C;
-    const size_t need = sel_layout(h, n_loc, k_max, C, true, multi).total;
-    if (n_loc + 1 <= 128 && need <= kSmemBudget) {  // the dims-major logits take <= 128 columns
-      *keys_in_smem = true;
-      *smem_bytes = need;
-      return C;
-    }
+    *smem_bytes = sel_layout(h, n_loc, k_max, C, true, multi).total;
+    return n_loc + 1 <= 128 && *smem_bytes <= kSmemBudget;  // the dims-major logits take <= 128 columns
+  };
+  auto stream = [&]() { *smem_bytes = sel_layout(h, (n_max + 15) / 16, k_max, 16, false, multi).total; };
+  if (multi) {  // (keys streamed by 16 CTAs cost a deep round less than keys held by 8)
+    *keys_in_smem = keys_fit(16);
+    if (!*keys_in_smem) stream();
+    if (wide_clusters_fit(bd.ep_off[bd.B], h, *smem_bytes)) return 16;
   }
+  *keys_in_smem = true;
+  for (int C : {8, 16})
+    if (keys_fit(C)) return C;
   *keys_in_smem = false;
-  *smem_bytes = sel_layout(h, (n_max + 15) / 16, k_max, 16, false, multi).total;
+  stream();
   return 16;
 }
 
@@ -1293,7 +1331,7 @@ cudaError_t select_launch(const BatchDesc& bd, int n_episodes, const SelectArgs&
   }
   const int n_loc = (n_max + C - 1) / C;
   const SelSmem L = sel_layout(a.h, n_loc, a.k_max, C, keys_in_smem, a.n_dec > 1);
-  void (*kern)(const BatchDesc, const SelectArgs, int, int, int) = nullptr;
+  SelectKernel kern = nullptr;
   const int gl = a.g + 1 <= 2 ? 2 : (a.g + 1 <= 6 ? 6 : 17);
   const bool train = a.score != nullptr;
   if (train && (a.g != 1 || !keys_in_smem || !a.kbar)) return cudaErrorInvalidValue;
@@ -1301,7 +1339,7 @@ cudaError_t select_launch(const BatchDesc& bd, int n_episodes, const SelectArgs&
   if (multi && (a.g != 1 || train || !a.dec || !a.dcache || !a.KC)) return cudaErrorInvalidValue;
 #define SP_SEL_CASE(HV_)                                                                                    \
   case HV_:                                                                                                 \
-    kern = multi ? select_kernel<HV_, 2, false, true>                                                       \
+    kern = multi ? deep_kernel(a.h)                                                                         \
                  : train ? select_kernel<HV_, 2, true, false>                                               \
                          : (gl == 2 ? select_kernel<HV_, 2, false, false>                                   \
                                     : (gl == 6 ? select_kernel<HV_, 6, false, false>                        \

@@ -102,6 +102,29 @@ def test_deep_decoder_llava_shapes(B):
     print("kept", gpu["count"].tolist(), "near-tie episodes", near)
 
 
+def test_deep_decoder_episodes_run_at_once(B):
+    """Eight episodes have room beside one another: they take no more than half as long again as four (twice as
+    long where their clusters would run in two waves)."""
+    w = _with_layers(S.tiny_workload(75, [64], [1], D=128, h=128, k_max=16), 2)
+    sel = _deep_weights(w, 4.0)
+    shape = S.SelectorShape(D=128, D_text=w.selector.D_text, h=128, n_enc_layers=0, n_dec_layers=2)
+    selector = B.Selector(shape, sel, DEV)
+    best = {}
+    for e in (4, 8):
+        H = B.dev_f32(np.concatenate([S.make_memory(w)] * e), DEV)
+        bias, ws, times = B.dev_f32(np.full(e, -1e30, np.float32), DEV), None, []
+        for _ in range(12):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            ws = B.sp_select(selector, [64] * e, [1] * e, H=H, stop_bias=bias, k_max=16, ws=ws)["_ws"]
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(t0.elapsed_time(t1))
+        best[e] = min(times)
+    assert best[8] <= 1.5 * best[4], best
+    selector.close()
+
+
 def test_deep_decoder_rejects_groups_of_tokens_per_round(B):
     w = _with_layers(S.tiny_workload(74, [20], [1], D=128, h=128, k_max=8), 2)
     sel = _deep_weights(w, 4.0)
