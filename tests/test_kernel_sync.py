@@ -35,7 +35,7 @@ def test_cluster_barrier_before_the_first_round(name, kernel):
     """Kernels that write into other CTAs' shared memory wait for the whole cluster to have started first: a
     cluster barrier on every path before the first round."""
     statements = _top_level(_source(name), kernel, "while (nsel < k_max)")
-    assert re.search(r"(^|;|\})\s*cluster\.sync\(\);", statements), "a CTA may write to a peer that has not started"
+    assert re.search(r"(^|;|\})\s*(cluster\.sync|cluster_sync_all)\(\);", statements), "a CTA may write to a peer that has not started"
 
 
 def test_warp_waits_order_the_other_lanes():
