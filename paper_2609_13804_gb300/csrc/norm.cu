@@ -331,10 +331,11 @@ assemble_wide_kernel(const BatchDesc bd, const __nv_bfloat16* X, const float* P,
 // sources: the encoder's residual R, the given memory H, or the visual tokens X
 // themselves) as the split operand of the precompute GEMM: [rows, 2D] fp16
 // (parts a1 | a2 of the scaled row) with the inverse scales, or [rows, 3D] bf16
-// (PARTS = 3); optionally the visual rows go to `memory` (fp32).  HBM-bound, a
-// warp per row.  NV > 0: all of the row's 16-byte loads in flight, the row held
-// in registers (NV float4 per lane) between the search for its largest element
-// and the split; NV = 0 (rows wider than that): read twice for PARTS = 2.
+// (PARTS = 3, always where D > kSplit2MaxD); optionally the visual rows go to
+// `memory` (fp32).  HBM-bound, a warp per row.  NV > 0: all of the row's 16-byte
+// loads in flight, the row held in registers (NV float4 per lane), for PARTS = 2
+// between the search for its largest element and the split; NV = 0: rows wider
+// than that.
 template <int NV, int PARTS>
 __global__ void __launch_bounds__(NT)
 memory_split_kernel(const BatchDesc bd, const float* R, const float* H, const uint2* X, const float* s_stop,
@@ -391,27 +392,27 @@ memory_split_kernel(const BatchDesc bd, const float* R, const float* H, const ui
       }
     }
   };
-  float m = 0.f, iv;
   if constexpr (NV > 0) {
     float4 v[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k)
       if (lane + 32 * k < n4) v[k] = load(lane + 32 * k);
+    float sc = 1.f;
+    if constexpr (PARTS == 2) {
+      float m = 0.f, iv;
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-      if (lane + 32 * k < n4) m = fmaxf(m, max_abs4(v[k]));
-    const float sc = split_scale(warp_max(m), &iv);
+      for (int k = 0; k < NV; ++k)
+        if (lane + 32 * k < n4) m = fmaxf(m, max_abs4(v[k]));
+      sc = split_scale(warp_max(m), &iv);
+      if (lane == 0) inv[r] = iv;
+    }
 #pragma unroll
     for (int k = 0; k < NV; ++k)
       if (lane + 32 * k < n4) put(lane + 32 * k, v[k], sc);
   } else {
 #pragma unroll 4
-    for (int i = PARTS == 2 ? lane : n4; i < n4; i += 32) m = fmaxf(m, max_abs4(load(i)));
-    const float sc = split_scale(warp_max(m), &iv);
-#pragma unroll 4
-    for (int i = lane; i < n4; i += 32) put(i, load(i), sc);
+    for (int i = lane; i < n4; i += 32) put(i, load(i), 1.f);
   }
-  if (PARTS == 2 && lane == 0) inv[r] = iv;
 }
 
 // LN1 of the decoder tokens (rows of h floats, ldx apart) as the split operand of
@@ -470,17 +471,20 @@ static bool aligned16(const void* a, const void* b) {
   return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
 }
 
-// Calls f(float4 per lane) with the register form of a row of d floats.
-template <class F>
+constexpr int kRowFormMax = 4096;  // widest row of the register form (32 float4 per lane)
+
+// Calls f(float4 per lane) with the register form of a row of d <= MAX floats.
+template <int MAX = kRowFormMax, class F>
 static cudaError_t with_row_form(int d, F f) {
+  if (d > MAX) return cudaErrorInvalidValue;
   if (d <= 256) return f(std::integral_constant<int, 2>{});
   if (d <= 512) return f(std::integral_constant<int, 4>{});
-  if (d <= 1024) return f(std::integral_constant<int, 8>{});
-  if (d <= 2048) return f(std::integral_constant<int, 16>{});
-  return f(std::integral_constant<int, 32>{});
+  if (MAX <= 1024 || d <= 1024) return f(std::integral_constant<int, 8>{});
+  if constexpr (MAX > 1024) {
+    if (MAX <= 2048 || d <= 2048) return f(std::integral_constant<int, 16>{});
+    if constexpr (MAX > 2048) return f(std::integral_constant<int, 32>{});
+  }
 }
-
-constexpr int kRowFormMax = 4096;  // widest row of the register form (32 float4 per lane)
 
 static int row_blocks(int rows) { return (rows + NT / 32 - 1) / (NT / 32); }
 
@@ -505,9 +509,9 @@ cudaError_t layernorm_bf16(const float* x, const float* gain, const float* bias,
 cudaError_t layernorm_split(const float* x, int ldx, const float* gain, const float* bias, void* out, float* inv,
                             int rows, int d, float eps, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  if (d > 1024 || d % 4 != 0 || ldx % 4 != 0) return cudaErrorInvalidValue;
+  if (d % 4 != 0 || ldx % 4 != 0) return cudaErrorInvalidValue;
   prof_begin_launch(st);
-  const cudaError_t r = with_row_form(d, [&](auto nv) {
+  const cudaError_t r = with_row_form<1024>(d, [&](auto nv) {
     return launch_pdl(layernorm_split_kernel<decltype(nv)::value>, dim3(row_blocks(rows)), dim3(NT), 0, st, x, ldx,
                       gain, bias, aligned16(gain, bias) ? 1 : 0, static_cast<uint2*>(out), inv, rows, d / 4, eps);
   });
@@ -563,13 +567,18 @@ cudaError_t memory_split(const BatchDesc& bd, const float* R, const float* H, co
                          const float* s_start, void* out, float* inv, float* memory, int D, cudaStream_t st) {
   const int rows = bd.vis_off[bd.B] + 2;
   prof_begin_launch(st);
-  auto go = [&](auto nv) {
-    constexpr int NV = decltype(nv)::value;
-    return launch_pdl(inv ? memory_split_kernel<NV, 2> : memory_split_kernel<NV, 3>, dim3(row_blocks(rows)), dim3(NT), 0, st, bd, R, H,
-                      static_cast<const uint2*>(X), s_stop, s_start, static_cast<uint2*>(out), inv, memory, D / 4, rows,
-                      aligned16(s_stop, s_start) ? 1 : 0, aligned16(memory, nullptr) ? 1 : 0);
+  auto go = [&](auto kern) {
+    return launch_pdl(kern, dim3(row_blocks(rows)), dim3(NT), 0, st, bd, R, H, static_cast<const uint2*>(X), s_stop,
+                      s_start, static_cast<uint2*>(out), inv, memory, D / 4, rows, aligned16(s_stop, s_start) ? 1 : 0,
+                      aligned16(memory, nullptr) ? 1 : 0);
   };
-  const cudaError_t r = D <= kRowFormMax ? with_row_form(D, go) : go(std::integral_constant<int, 0>{});
+  cudaError_t r;
+  if (inv)
+    r = with_row_form<2048>(D, [&](auto nv) { return go(memory_split_kernel<decltype(nv)::value, 2>); });
+  else if (D <= kRowFormMax)
+    r = with_row_form(D, [&](auto nv) { return go(memory_split_kernel<decltype(nv)::value, 3>); });
+  else
+    r = go(memory_split_kernel<0, 3>);
   prof_end_launch(st, SP_K_SGEMM, 0.0, (memory ? 12.0 : 8.0) * rows * (double)D);
   return r;
 }
