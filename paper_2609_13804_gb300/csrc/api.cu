@@ -459,12 +459,16 @@ struct SelPlan {
 
 size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* out, Carve& cv, void** parts);
 
-// Whether the selection goes through per-episode tables.  They cost kGramFixedUs
-// and 30 h (n + 2)^2 tensor operations per episode (16 x 576 candidates, h = 512:
-// 140 us with their operands, 0.59e9 a microsecond; one of 576, h = 256: 23 us)
-// and save kGramRoundUs of every round (16 x 576: 4.9 -> 2.5 us; training 6.8 ->
-// 2.6; one image 5.6 -> 2.1); the rounds are bounded by the cap (a STOP can end
-// them early, which only the device knows).
+// Whether the selection goes through per-episode tables.  They are taken to cost
+// kGramFixedUs and 30 h (n + 2)^2 tensor operations per episode (measured, 576
+// candidates with h = 512: 1, 4, 8, 14, 16 images 11, 49, 79, 128, 136 us) and to
+// save kGramRoundUs of every round (measured: 14 such images 5.9 -> 2.9 us, one
+// 5.7 -> 2.5, one with h = 256 5.2 -> 2.5, 8 with the training aggregates 7.0 ->
+// 3.4).  Waves are not counted: 16 images are one more than a card with room for
+// 15 clusters of 8 runs at once and save 12.1 -> 5.3 us a round, and 64, with
+// 192 rounds, would gain but stay with the general kernel.  The rounds are
+// bounded by the cap; a STOP, which only the device knows, can end them before
+// the tables have paid (the first 20 rounds for those 16 images, 4 for one).
 constexpr double kGramFixedUs = 15.0;
 constexpr double kGramOpsPerUs = 0.55e9;
 constexpr double kGramRoundUs = 2.5;
@@ -484,7 +488,10 @@ void plan_gram(const sp_selector* s, const sp_select_in* in, SelPlan* p) {
   if (C == 0) return;
   gram_layout(p->E, p->nvis, p->n_max, h, &p->gram);
   // A batch that the allocation-free entry point takes runs the same way with
-  // a caller's workspace: tables only if they fit its scratch too.
+  // a caller's workspace (the same kernels, so the same traces to the bit): tables
+  // only if they fit its scratch too.  From a given memory of D = 1,024 that
+  // leaves 5 x 576 candidates, h = 512, with the general kernel: 192 rounds in
+  // 1,191 us, where 4 x 576 take 561.
   Carve base(nullptr), full(nullptr);
   const size_t b0 = select_ws(s, *p, nullptr, base, nullptr) + 256;
   p->gram_C = C;
@@ -531,9 +538,9 @@ size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* ou
   } else if (p.encoder) {
     R = cv.take<float>((size_t)p.T_enc * D);
   }
-  // (the first two are unused by the general kernel: the size that callers' workspaces and the
-  // allocation-free entry point's limit are checked against stays what it was when the memory and its LN1
-  // were stored in fp32; the tables' operands take the place of all three after the precompute)
+  // (the first two, and R without encoder blocks, are unused by the general kernel: the size that callers'
+  // workspaces and the allocation-free entry point's limit are checked against stays what it was when the memory
+  // and its LN1 were stored in fp32; the tables' operands take the place of these three after the precompute)
   void* op = cv.take<float>((size_t)p.rows * D);
   const size_t op0 = cv.off - (size_t)p.rows * D * sizeof(float);
   cv.take<float>((size_t)p.rows * h);
@@ -555,8 +562,8 @@ size_t select_ws(const sp_selector* s, const SelPlan& p, const sp_select_out* ou
   float* dcache = s->n_dec > 1 ? cv.take<float>((size_t)p.E * (s->n_dec - 1) * (p.k_max + 1) * 2 * h) : nullptr;
   if (parts) {
     parts[0] = P; parts[1] = R; parts[2] = Abf; parts[3] = QKV; parts[4] = O; parts[5] = F1;
-    parts[6] = enc_cu; parts[7] = op; parts[8] = ZK; parts[9] = nullptr; parts[10] = QKVs;
-    parts[11] = order; parts[12] = epc; parts[13] = gsk; parts[14] = Asp; parts[15] = dcache;
+    parts[6] = enc_cu; parts[7] = op; parts[8] = ZK; parts[9] = Asp; parts[10] = QKVs;
+    parts[11] = order; parts[12] = epc; parts[13] = gsk; parts[14] = dcache;
   }
   return cv.off;
 }
@@ -663,7 +670,7 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
   }
   if (out->k_cap < need_cap) return fail(SP_ERR_SHAPE, "sp_select: k_cap %d < largest possible count %d", out->k_cap, need_cap);
   Carve cv(ws);
-  void* parts[16];
+  void* parts[15];
   size_t need = select_ws(s, p, out, cv, parts) + 256;
   if (ws && ws_bytes < need && p.gram_C) {  // without room for the tables: the general kernel
     p.gram_C = 0;
@@ -684,7 +691,7 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
     rs = run_encoder(s, in, p, parts, err, st);
     if (rs != SP_OK) return rs;
   }
-  void* Asp = parts[14];
+  void* Asp = parts[9];
   const int parts1 = s->P1s && in->g == 1 ? 2 : 3;  // (precompute.cu)
   // the rows' inverse scales, behind the widest operand's two parts
   float* Ainv = reinterpret_cast<float*>(static_cast<uint16_t*>(Asp) + (size_t)p.rows * 2 * std::max(D, h));
@@ -695,7 +702,7 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
   float* QKVs = (float*)parts[10];
   // candidate precompute (fp32): [z | KT] = M [W_in; Wq_p^T Wk_p / sqrt h]^T, x = LN1(z),
   // [QS | KS | VT] = x [Wq_s / sqrt h; Wk_s; Wo_s Wv_s]^T
-  // (fp32-accurate products on the fp16 tensor cores: two-way operand split)
+  // (fp32-accurate products on the tensor cores: operand split, precompute.cu)
   {
     std::string msg;
     CUtensorMap t1, t2;
@@ -747,7 +754,7 @@ static sp_status select_impl(const sp_selector* s, const sp_select_in* in, const
   a.n_dec = s->n_dec;
   a.dec = s->dec_dev;
   a.KC = ZK + 2 * h;
-  a.dcache = static_cast<float*>(parts[15]);
+  a.dcache = static_cast<float*>(parts[14]);
   a.dcache_ep = (size_t)(s->n_dec - 1) * (in->k_max + 1) * 2 * h;
   bool keys_smem = true;
   size_t smem = 0;

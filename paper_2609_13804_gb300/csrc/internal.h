@@ -272,7 +272,7 @@ struct GramArgs {
   float* inv;              // [5][rows] inverse scales
   float* dj;               // [rows] <kt, ln2 bias>
   float* zz;               // [rows] |zc|^2
-  float* table;            // [E][ep_stride]
+  float* table;            // [E][ep_stride]; STOP's row, which nothing else reads, holds select_gram.cu's flag
   int* err;
 };
 void gram_layout(int E, int nvis, int n_max, int h, GramArgs* g);

@@ -24,12 +24,16 @@
 // product in three bf16 parts (x = x0 + x1 + x2, |r| <= 2^-24 |x|) as six
 // segments,
 //   A segments [a0 a0 a1 a0 a1 a2]  x  B segments [b0 b1 b0 b2 b1 b0].
-// That form's own rounding is the larger one (1.1e-5 of a logit at D = 1,024,
-// 3.8e-5 at 3,584, against 1.2e-6 and 3.9e-6 for two parts), and the margins of
-// grouped rounds are differences of neighbouring logits: they would move by up
-// to 5e-4 of themselves, where recorded traces are held to 1.5e-4.  With g = 1
-// the two forms' margins agree to 2e-5 and the faster one is used: 9,218 rows
-// of D = 1,024 in the two products: 140 -> 78 us.
+// No limit of the hardware stands behind this: that form is the slower one and
+// its own rounding the larger (1.1e-5 of a logit at D = 1,024, 3.8e-5 at 3,584,
+// against 1.2e-6 and 3.9e-6 for two parts; 9,218 rows of D = 1,024 in the two
+// products 140 us against 78).  It keeps results comparable: the margins of
+// grouped rounds are differences of neighbouring logits, and under two parts
+// they differ by up to 5e-4 of themselves from those of earlier versions, where
+// the measured cases allow 1.5e-4; with g = 1 the two forms' margins agree to
+// 2e-5.  So the same image with g = 1 and with g = 5 has logits that differ by
+// 1e-5, and a selector holds the weights in both forms.  Whoever can do without
+// the comparison replaces the three parts by two everywhere.
 #include <algorithm>
 
 #include "common.cuh"

@@ -29,9 +29,10 @@
 // general kernel has six, two and two and reads its whole key slice from
 // shared memory.  Latency-bound: the steps form one serial chain.  The margin
 // trace (the second best logit) is worked out in the shadow of the next loads.
-// Per round on GB300, general kernel -> here: 16 episodes of 576 with h = 512, up
-// to 192 rounds, 6.1 -> 2.5 us; 8 with the training aggregates, 96 rounds, 6.8 ->
-// 2.6; one with h = 256, 64 rounds, 5.6 -> 2.1.
+// Per round on GB300, general kernel -> here (rounds 97 to 192): 14 episodes of
+// 576 with h = 512 5.9 -> 2.9 us, 4 of them 5.7 -> 2.4; 8 with the training
+// aggregates 7.0 -> 3.4; one with h = 256 5.2 -> 2.5; one with g = 5 10.2 -> 5.2.
+// (16 run in two waves of clusters on a card with room for 15: 12.1 -> 5.3.)
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -618,12 +619,8 @@ static int gram_history(int k_max, int n_max) { return std::min(k_max, n_max); }
 int select_gram_cluster(int n_max, int k_max, int g) {
   const int T = gram_history(k_max, n_max);
   if (T > kMaxHist) return 0;
-  for (int C : {8}) {
-    const int n_loc = (n_max + C - 1) / C;
-    if (n_loc > kMaxSlice) continue;
-    if (gram_smem(T, n_loc, C, g + 1).total <= kSmemBudget) return C;
-  }
-  return 0;
+  const int n_loc = (n_max + kMaxCluster - 1) / kMaxCluster;
+  return n_loc <= kMaxSlice && gram_smem(T, n_loc, kMaxCluster, g + 1).total <= kSmemBudget ? kMaxCluster : 0;
 }
 
 template <bool CAREFUL>
